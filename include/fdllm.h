@@ -35,8 +35,10 @@
  *     as FDLLM_ERR_NONFINITE.
  *   - All kernels are deterministic: the same inputs on the same GPU model give
  *     bit-identical outputs.  A position's confidence depends only on its logits and the
- *     call's shape (B * L, V, dtype), which fix how rows are cut into reduction units, so
- *     identical rows of one call give identical confidences (exact ties stay ties).
+ *     call's shape (B * L, V, dtype), which fix how rows are cut into reduction units (in a
+ *     workspace smaller than the shape's fdllm_workspace_bytes that still holds one partial
+ *     per row, a row of at most 64 KB is one unit), so identical rows of one call give
+ *     identical confidences (exact ties stay ties).
  *   - Arithmetic: confidences are reduced in fp32 (relative error within 1e-5 of the exact
  *     value); the rules are evaluated on those fp32 confidences with exact 64-bit fixed-point
  *     prefix sums of 1 - c in units of 2^-52 (delta = 1 - f formed from the same integer as

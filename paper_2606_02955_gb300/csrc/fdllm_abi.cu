@@ -27,15 +27,26 @@ struct Layout {
     UnitPlan plan;
 };
 
-Layout layout_for(int64_t rows, int64_t row_bytes)
+Layout layout_for(int64_t rows, int64_t row_bytes, bool warp_units = true)
 {
     Layout l;
-    l.plan = plan_units(row_bytes, rows);
+    l.plan = plan_units(row_bytes, rows, warp_units);
     l.status = 0;
     l.next_unit = 4;
     l.partials = kAlign;
     l.total = align_up(l.partials + (size_t)rows * l.plan.units_per_row * sizeof(UnitPartial));
     return l;
+}
+
+// layout_for, or the layout of CTA units where only that one fits in `have` bytes: a workspace
+// sized for a longer vocabulary (at least one partial per row) keeps serving shorter ones.
+Layout layout_within(int64_t rows, int64_t row_bytes, size_t have)
+{
+    const Layout l = layout_for(rows, row_bytes);
+    if (l.total <= have)
+        return l;
+    const Layout c = layout_for(rows, row_bytes, false);
+    return c.total <= have ? c : l;
 }
 
 bool valid_dtype(int d) { return d == FDLLM_BF16 || d == FDLLM_FP32 || d == FDLLM_FP16; }
@@ -110,6 +121,24 @@ fdllm_status owned_workspace(size_t need, cudaStream_t stream, void **out)
 
 namespace {
 
+// The layout of a call on the library-owned workspace, which grows to hold it.  It cannot grow
+// while `stream` is captured: what fits the workspace as it is serves there.
+Layout owned_layout(int64_t rows, int64_t row_bytes, cudaStream_t stream)
+{
+    const Layout l = layout_for(rows, row_bytes);
+    size_t have = 0;
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices) {
+        std::lock_guard<std::mutex> lock(g_ws_mutex);
+        have = g_ws[dev].bytes;
+    }
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (l.total <= have || cudaStreamIsCapturing(stream, &cap) != cudaSuccess ||
+        cap == cudaStreamCaptureStatusNone)
+        return l;
+    return layout_within(rows, row_bytes, have);
+}
+
 VocabReduceArgs reduce_args(const void *logits, int dtype, int B, int L, int V,
                             const uint8_t *mask, uint8_t *ws, const Layout &lay)
 {
@@ -121,6 +150,7 @@ VocabReduceArgs reduce_args(const void *logits, int dtype, int B, int L, int V,
     a.vec_per_row = a.row_bytes / 16;
     a.units_per_row = lay.plan.units_per_row;
     a.unit_vecs = lay.plan.unit_vecs;
+    a.warp_units = lay.plan.warp_units;
     a.partials = reinterpret_cast<UnitPartial *>(ws + lay.partials);
     a.next_unit = reinterpret_cast<uint32_t *>(ws + lay.next_unit);
     a.status = reinterpret_cast<uint32_t *>(ws + lay.status);
@@ -242,7 +272,7 @@ fdllm_status select_owned(const void *logits, int dtype, int B, int L, int V, ui
                                         out_commit, out_n);
     if (st != FDLLM_OK)
         return st;
-    const Layout lay = layout_for((int64_t)B * L, (int64_t)V * esize_of(dtype));
+    const Layout lay = owned_layout((int64_t)B * L, (int64_t)V * esize_of(dtype), stream);
     void *ws = nullptr;
     st = owned_workspace(lay.total, stream, &ws);
     if (st != FDLLM_OK)
@@ -273,7 +303,8 @@ fdllm_status fdllm_select_ws(const void *logits, int dtype, int B, int L, int V,
                                         out_commit, out_n);
     if (st != FDLLM_OK)
         return st;
-    const Layout lay = layout_for((int64_t)B * L, (int64_t)V * esize_of(dtype));
+    const Layout lay =
+        layout_within((int64_t)B * L, (int64_t)V * esize_of(dtype), workspace_bytes);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) % kAlign) != 0 ||
         workspace_bytes < lay.total)
         return FDLLM_ERR_WORKSPACE;
@@ -301,8 +332,8 @@ fdllm_status fdllm_select_robust(const void *logits, int dtype, int B, int L, in
         return st;
     if (!std::isfinite(eta) || eta < 0.0)
         return FDLLM_ERR_ARG;
-    const Layout lay = layout_for((int64_t)B * L, (int64_t)V * esize_of(dtype));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const Layout lay = owned_layout((int64_t)B * L, (int64_t)V * esize_of(dtype), s);
     void *ws = nullptr;
     st = owned_workspace(lay.total, s, &ws);
     if (st != FDLLM_OK)
@@ -349,8 +380,8 @@ fdllm_status fdllm_confidence(const void *logits, int dtype, int B, int L, int V
         return st;
     if (!plan_fits((int64_t)B * L, (int64_t)V * esize_of(dtype)))
         return FDLLM_ERR_ARG;
-    const Layout lay = layout_for((int64_t)B * L, (int64_t)V * esize_of(dtype));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const Layout lay = owned_layout((int64_t)B * L, (int64_t)V * esize_of(dtype), s);
     void *ws = nullptr;
     st = owned_workspace(lay.total, s, &ws);
     if (st != FDLLM_OK)
@@ -385,8 +416,8 @@ fdllm_status fdllm_vocab_reduce(const void *logits, int dtype, int B, int L, int
         return st;
     if (!plan_fits((int64_t)B * L, (int64_t)V * esize_of(dtype)))
         return FDLLM_ERR_ARG;
-    const Layout lay = layout_for((int64_t)B * L, (int64_t)V * esize_of(dtype));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const Layout lay = owned_layout((int64_t)B * L, (int64_t)V * esize_of(dtype), s);
     void *ws = nullptr;
     st = owned_workspace(lay.total, s, &ws);
     if (st != FDLLM_OK)

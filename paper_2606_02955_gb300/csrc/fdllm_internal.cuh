@@ -19,9 +19,8 @@ namespace fdllm {
 // shared-memory chunk buffers.  The target is 128 KB; a step whose logits, all B * L rows
 // counted, fit in about one wave of such units over the SMs (kSmallStepBytes) takes 64 KB
 // units instead, so that twice as many SMs share its reduction: there the per-SM exp
-// throughput and the first copy's latency, not HBM, set the time.  Smaller units pay for
-// themselves nowhere: a unit must fill the ring (192 KB in flight per SM) to stream at
-// full bandwidth.
+// throughput and the first copy's latency, not HBM, set the time.  A smaller unit does not
+// fill the ring (192 KB in flight per SM), so short rows take warp units (below).
 constexpr int kSegQueue = 8;  // unit results queued from math warps to the epilogue warp
 constexpr int64_t kUnitTargetBytes = 131072;
 constexpr int64_t kSmallUnitTargetBytes = 65536;
@@ -56,11 +55,13 @@ struct VocabReduceArgs {
                              // zero again after the launch's last fetch
     uint32_t *status;        // sticky device error bits
     bool pdl = true;         // launch as a programmatic dependent of the previous kernel
+    bool warp_units = false; // the units are warp units (UnitPlan)
 };
 
 struct UnitPlan {
     int32_t units_per_row;
     int32_t unit_vecs;
+    bool warp_units;  // one warp reduces a unit, otherwise one CTA
 };
 
 // Unit lengths are rounded up to a multiple of kUnitAlignVecs vectors (8 KB), so that every
@@ -68,9 +69,36 @@ struct UnitPlan {
 // no unit is empty.
 constexpr int64_t kUnitAlignVecs = 512;
 
-inline UnitPlan plan_units(int64_t row_bytes, int64_t rows)
+// Short rows.  A unit reduced by a whole CTA pays a ring hand-over and a 16-warp reduction
+// (about 1.4 us) and has only itself in flight, so where a row is one unit of at most 64 KB
+// the units are warp units instead: one warp each, 32 in flight per SM.  Measured per launch,
+// CTA units against warp units: 1004 fp32 logits x 44100 rows 403 against 34 us, 4096 bf16 x
+// 6554 rows 66 against 14, 20008 fp16 x 6393 rows 67 against 42, 32000 bf16 x 1434 rows 19.1
+// against 19.0 (level: the bound on the row), 50304 bf16 x 1434 rows 28.9 against 29.0, and
+// 50304 fp32 x 1434 rows 43.9 against 47.0.  With at most two rows per SM a CTA spreads a
+// row over more lanes: 20008 bf16 x 32 rows 4.1 against 5.6 us, x 205 rows 6.6 against 6.4.
+// 8 KB units measured fastest (128, 256, 512 and 1024 vectors: 50.2, 50.2, 42.2 and 44.3 us at
+// 20008 fp16), and at most 8 of them let one thread fold a position's partials in one round.
+constexpr int64_t kWarpRowBytes = 65536;
+constexpr int64_t kWarpMinRows = 2 * 152;
+constexpr int64_t kWarpUnitVecs = 512;
+static_assert(kWarpRowBytes / 16 / kWarpUnitVecs <= 8, "partials folded in one round");
+
+// warp_units = false plans CTA units whatever the shape: one partial per short row, for scratch
+// memory that does not hold more (see layout_within).
+inline UnitPlan plan_units(int64_t row_bytes, int64_t rows, bool warp_units = true)
 {
     const int64_t vpr = row_bytes / 16;
+    if (warp_units && row_bytes <= kWarpRowBytes && rows > kWarpMinRows) {
+        // no more units than the static scratch array has room for
+        const int64_t fit =
+            (FDLLM_STATIC_SCRATCH_BYTES - 256) / (int64_t)sizeof(UnitPartial) / rows;
+        int64_t upr = (vpr + kWarpUnitVecs - 1) / kWarpUnitVecs;
+        upr = upr > fit ? fit : upr;
+        upr = upr < 1 ? 1 : upr;
+        const int64_t uv = ((vpr + upr - 1) / upr + 31) / 32 * 32;
+        return UnitPlan{(int32_t)((vpr + uv - 1) / uv), (int32_t)uv, true};
+    }
     const int64_t target =
         rows * row_bytes <= kSmallStepBytes ? kSmallUnitTargetBytes : kUnitTargetBytes;
     int64_t upr = (row_bytes + target - 1) / target;
@@ -81,7 +109,7 @@ inline UnitPlan plan_units(int64_t row_bytes, int64_t rows)
     upr = (vpr + uv - 1) / uv;
     if (upr < 1)
         upr = 1;
-    return UnitPlan{(int32_t)upr, (int32_t)uv};
+    return UnitPlan{(int32_t)upr, (int32_t)uv, false};
 }
 
 // Enqueue the vocab reduction on all SMs, as a programmatic dependent of the previous

@@ -705,6 +705,245 @@ __global__ void __launch_bounds__((NW + 2) * 32, 1) vocab_reduce_kernel(const Vo
     }
 }
 
+// ------------------------------------------------------------------ short rows (warp units)
+// A launch whose units are warp units (UnitPlan::warp_units): one warp reduces one unit with
+// plain 16-byte loads, kWarpBatch of them in flight per lane, and 32 such warps per SM keep
+// 128 KB in flight whatever the rows' length.
+constexpr int kUnitWarps = 32;
+constexpr int kWarpBatch = 8;  // 16-byte vectors per lane and batch: 4 KB per warp
+
+// One 16-byte vector of the stream: read once, first to evict.
+__device__ __forceinline__ uint4 load_stream(const uint4 *p)
+{
+    return __ldcs(p);
+}
+
+template <int KIND>
+__global__ void __launch_bounds__(kUnitWarps * 32, 1)
+    vocab_warp_units_kernel(const VocabReduceArgs a)
+{
+    using Ops = VecOps<KIND>;
+    constexpr int kP = Ops::kPairs;
+    extern __shared__ uint16_t s_rows[];  // this CTA's masked rows, ascending
+    __shared__ uint32_t s_warp[kUnitWarps];
+    __shared__ uint32_t s_next;
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    constexpr uint32_t kFull = 0xFFFFFFFFu;
+
+    pdl_wait();  // the mask and the logits are written
+    if (threadIdx.x == 0)
+        pdl_launch_dependents();
+
+    // The masked rows counted, each thread `per` (a multiple of 16) consecutive rows.
+    const int rows = (int)a.rows;
+    const int per = ((rows + kUnitWarps * 32 - 1) / (kUnitWarps * 32) + 15) & ~15;  // <= 64
+    const int row0 = (int)threadIdx.x * per;
+    uint64_t bits = 0;
+    if (row0 < rows) {
+        if ((reinterpret_cast<uintptr_t>(a.mask) & 15u) == 0 && row0 + per <= rows) {
+            uint4 v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (16 * i < per)
+                    v[i] = __ldcg(reinterpret_cast<const uint4 *>(a.mask + row0 + 16 * i));
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (16 * i < per)
+                    bits |= (uint64_t)(nonzero_bytes4(v[i].x) | (nonzero_bytes4(v[i].y) << 4) |
+                                       (nonzero_bytes4(v[i].z) << 8) |
+                                       (nonzero_bytes4(v[i].w) << 12))
+                            << (16 * i);
+        } else {
+            for (int i = 0; i < per && row0 + i < rows; ++i)
+                bits |= (uint64_t)(a.mask[row0 + i] != 0 ? 1u : 0u) << i;
+        }
+    }
+    const uint32_t cnt = (uint32_t)__popcll(bits);
+    uint32_t incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o)
+            incl += t;
+    }
+    if (lane == 31)
+        s_warp[warp] = incl;
+    __syncthreads();
+    const uint32_t wsum = s_warp[lane];
+    uint32_t wincl = wsum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, wincl, o);
+        if (lane >= o)
+            wincl += t;
+    }
+    const uint32_t masked = __shfl_sync(kFull, wincl, 31);
+    const uint32_t before = __shfl_sync(kFull, wincl - wsum, warp);
+
+    // This CTA's share of the units, and the rows they belong to.
+    const uint32_t upr = (uint32_t)a.units_per_row;
+    const uint64_t total = (uint64_t)masked * upr;
+    const uint32_t u0 = (uint32_t)(total * blockIdx.x / gridDim.x);
+    const uint32_t u1 = (uint32_t)(total * (blockIdx.x + 1) / gridDim.x);
+    if (u0 == u1)
+        return;
+    const uint32_t r0 = u0 / upr, r1 = (u1 + upr - 1) / upr;
+    uint32_t rank = before + incl - cnt;
+    if (rank < r1 && rank + cnt > r0)
+        while (bits != 0) {
+            const int b = __ffsll((long long)bits) - 1;
+            bits &= bits - 1;
+            if (rank >= r0 && rank < r1)
+                s_rows[rank - r0] = (uint16_t)(row0 + b);
+            ++rank;
+        }
+    if (threadIdx.x == 0)
+        s_next = u0 + kUnitWarps;
+    __syncthreads();
+
+    // A warp's units, batch by batch.  The next batch (of this unit, or the first one of the
+    // warp's next unit) is loaded before a finished unit's lanes are reduced, so the reduction's
+    // latency is hidden behind the loads.
+    const uint4 pad = make_uint4(Ops::kPadWord, Ops::kPadWord, Ops::kPadWord, Ops::kPadWord);
+    struct Unit {
+        const uint4 *src;
+        uint32_t n;      // vectors; 0: no unit
+        uint32_t vbase;  // row-relative index of its first vector
+        uint32_t slot;   // partial slot
+    };
+    auto locate = [&](uint32_t u) {
+        Unit x{nullptr, 0, 0, 0};
+        if (u < u1) {
+            const uint32_t r = u / upr, j = u - r * upr;
+            const uint32_t row = s_rows[r - r0];
+            x.vbase = j * (uint32_t)a.unit_vecs;
+            x.n = min((uint32_t)a.unit_vecs, (uint32_t)a.vec_per_row - x.vbase);
+            x.src = reinterpret_cast<const uint4 *>(a.logits + (int64_t)row * a.row_bytes) +
+                    x.vbase;
+            x.slot = row * upr + j;
+        }
+        return x;
+    };
+    uint4 raw[kWarpBatch];
+    auto load = [&](const uint4 *src, uint32_t n) {  // n vectors from src (at most a batch)
+        if (n >= kWarpBatch * 32) {
+#pragma unroll
+            for (int i = 0; i < kWarpBatch; ++i)
+                raw[i] = load_stream(src + i * 32 + lane);
+        } else {
+#pragma unroll
+            for (int i = 0; i < kWarpBatch; ++i)
+                if (i * 32 < n)
+                    raw[i] = i * 32 + lane < n ? load_stream(src + i * 32 + lane) : pad;
+        }
+    };
+
+    Unit cur = locate(u0 + warp);
+    if (cur.n == 0)
+        return;
+    load(cur.src, cur.n);
+    uint32_t v0 = 0;
+    float m = -INFINITY;  // lane max, propagating NaN
+    uint32_t best = 0;    // the lane's first vector attaining it (from the unit's start)
+    // The lane's own reference of rebase_scaled; before the first finite logit ref = -inf.
+    float ref = -INFINITY, ref2 = -FLT_MAX, sc = kLog2e;
+    uint64_t acc[kP];
+#pragma unroll
+    for (int q = 0; q < kP; ++q)
+        acc[q] = 0;
+    for (;;) {
+        const uint32_t rem = cur.n - v0;
+        float bm = Ops::vmax(raw[0]);
+        int bi = 0;
+#pragma unroll
+        for (int i = 1; i < kWarpBatch; ++i)
+            if (i * 32 < rem) {
+                const float t = Ops::vmax(raw[i]);
+                bi = t > bm ? i : bi;
+                bm = fmax_nan(bm, t);
+            }
+        best = bm > m ? v0 + bi * 32 + lane : best;
+        m = fmax_nan(m, bm);
+        if (m > ref + kRebaseSlack) {
+            const bool big = !(fabsf(m) < kBigRef);
+            const float r2 = big ? m : m * kLog2e;
+            const float f = (big || sc != kLog2e) ? 0.0f : ex2_mufu(ref2 - r2);
+            const uint64_t f2 = pack2(f, f);
+#pragma unroll
+            for (int q = 0; q < kP; ++q)
+                acc[q] = fmul2(acc[q], f2);
+            ref = m;
+            ref2 = r2;
+            sc = big ? 1.0f : kLog2e;
+        }
+        const uint64_t nref2 = pack2(-ref2, -ref2), sc2 = pack2(sc, sc);
+#pragma unroll
+        for (int i = 0; i < kWarpBatch; ++i)
+            if (i * 32 < rem) {
+                uint64_t p[kP];
+                Ops::pairs(raw[i], p);
+#pragma unroll
+                for (int q = 0; q < kP; ++q) {
+                    float t0, t1;
+                    unpack2(ffma2(p[q], sc2, nref2), t0, t1);
+                    acc[q] = fadd2(acc[q], pack2(ex2_mufu(t0), ex2_mufu(t1)));
+                }
+            }
+        v0 += kWarpBatch * 32;
+        if (v0 < cur.n) {
+            load(cur.src + v0, cur.n - v0);
+            continue;
+        }
+        uint32_t un = 0;
+        if (lane == 0)
+            un = atomicAdd(&s_next, 1u);
+        const Unit next = locate(__shfl_sync(kFull, un, 0));
+        load(next.src, next.n);
+
+        const float M = unordered(__reduce_max_sync(kFull, ordered(m)));
+        uint4 win = pad;
+        if (m == M)
+            win = __ldcg(cur.src + best);
+        float S = 0.0f;
+#pragma unroll
+        for (int q = 0; q < kP; ++q) {
+            float lo, hi;
+            unpack2(acc[q], lo, hi);
+            S += lo + hi;
+        }
+        S = rebase_scaled(S, sc, ref2, M);
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1)
+            S += __shfl_xor_sync(kFull, S, o);
+        const bool bad = __any_sync(kFull, m != m);
+        uint32_t idx = kNoIdx;
+        if (m == M)
+            idx = (cur.vbase + best) * Ops::kElems + Ops::first_index(win, M);
+        idx = __reduce_min_sync(kFull, idx);
+        if (lane == 0) {
+            UnitPartial p;
+            p.M = M;
+            p.S = bad ? __int_as_float(0x7FC00000) : (M == -INFINITY ? 0.0f : S);
+            p.idx = idx;
+            p.pad = 0;
+            a.partials[cur.slot] = p;
+        }
+        if (next.n == 0)
+            return;
+        cur = next;
+        v0 = 0;
+        m = -INFINITY;
+        best = 0;
+        ref = -INFINITY;
+        ref2 = -FLT_MAX;
+        sc = kLog2e;
+#pragma unroll
+        for (int q = 0; q < kP; ++q)
+            acc[q] = 0;
+    }
+}
+
 __global__ void finalize_kernel(const FinalizeArgs a)
 {
     pdl_wait();  // the vocab reduction's partials are complete and visible
@@ -782,6 +1021,36 @@ cudaError_t launch_kind(const VocabReduceArgs &a, cudaStream_t stream, int which
     }
 }
 
+template <int KIND>
+cudaError_t launch_warp_units(const VocabReduceArgs &a, cudaStream_t stream)
+{
+    static std::once_flag once[64];
+    static int sms[64];
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess)
+        return err;
+    if (dev < 0 || dev >= 64)
+        return cudaErrorInvalidDevice;
+    std::call_once(once[dev], [&] {
+        int n = 0;
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        sms[dev] = n < 8 ? 8 : n;  // (rows / 8 + 4) row ids stay within 48 KB
+    });
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)sms[dev]);
+    cfg.blockDim = dim3(kUnitWarps * 32);
+    // a CTA's units lie in at most ceil(rows / grid) + 1 rows
+    cfg.dynamicSmemBytes = (size_t)(a.rows / sms[dev] + 4) * sizeof(uint16_t);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, vocab_warp_units_kernel<KIND>, a);
+}
+
 int variant_index()
 {
     static const int v = [] {
@@ -811,6 +1080,12 @@ cudaError_t launch_bounded_wait_probe(uint32_t *status, uint64_t limit_ns, cudaS
 
 cudaError_t launch_vocab_reduce(const VocabReduceArgs &a, int dtype, cudaStream_t stream)
 {
+    if (a.warp_units)
+        switch (dtype) {
+        case FDLLM_BF16: return launch_warp_units<FDLLM_BF16>(a, stream);
+        case FDLLM_FP16: return launch_warp_units<FDLLM_FP16>(a, stream);
+        default: return launch_warp_units<FDLLM_FP32>(a, stream);
+        }
     const int which = variant_index();
     switch (dtype) {
     case FDLLM_BF16: return launch_kind<FDLLM_BF16>(a, stream, which);
