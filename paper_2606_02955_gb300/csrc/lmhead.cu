@@ -43,6 +43,10 @@ constexpr uint32_t kAccStride = 256;  // TMEM columns between the two accumulato
 constexpr uint32_t kTmemCols = 512;
 constexpr size_t kBarrierBytes = 256;
 constexpr size_t kRingBudget = 220 * 1024;
+// kStore: an epilogue warp's 32 x 32 block of logits on its way to memory, rows padded to 33 so
+// that writing it by column and reading it by row are both free of bank conflicts.
+constexpr int kStagePitch = 33;
+constexpr int kStageWarpFloats = 32 * kStagePitch;
 
 // How the CTAs of a cluster share a W tile.
 enum Mode {
@@ -60,21 +64,24 @@ constexpr int PAIR_KB = 2;  // pair mode: K-blocks per stage
 // stage count fills the ring budget: solo 4 x 48 KB at 256, 5 x 42 KB at 208; pair 3 x 64 KB
 // at 256 (each CTA holds half the W tile, and a stage two K-blocks: with the pair's two
 // cross-CTA signals per stage, fewer and larger stages measured faster than 6 x 32 KB).
-template <int BN_, int MODE>
+enum Epilogue { kReduce = 0, kStore = 1 };
+
+template <int BN_, int MODE, int EPI = kReduce>
 struct TileCfg {
     static constexpr int BN = BN_;
     static constexpr int kBRows = MODE == kPair ? BN / 2 : BN;  // W rows held per CTA
     static constexpr int kBBytes = kBRows * BK * 2;
     static constexpr int kKB = MODE == kPair ? PAIR_KB : 1;       // K-blocks of BK per stage
     static constexpr int kStageBytes = kKB * (kABytes + kBBytes);
-    static constexpr int kStages =
-        (int)(kRingBudget / kStageBytes) > 8 ? 8 : (int)(kRingBudget / kStageBytes);
-    static constexpr size_t kSmemBytes = 1024 + (size_t)kStages * kStageBytes + kBarrierBytes;
+    static constexpr size_t kStagingBytes = EPI == kStore ? 4 * kStageWarpFloats * 4 : 0;
+    static constexpr int kFit = (int)((kRingBudget - kStagingBytes) / kStageBytes);
+    static constexpr int kStages = kFit > 8 ? 8 : kFit;
+    static constexpr size_t kSmemBytes =
+        1024 + (size_t)kStages * kStageBytes + kBarrierBytes + kStagingBytes;
+    static_assert(kSmemBytes <= 227 * 1024, "ring and staging");
     static_assert(BN % 16 == 0 && BN <= (int)kAccStride, "MMA N");
     static_assert((BN / 2) % 8 == 0, "halves of whole 8-row swizzle atoms");
 };
-
-enum Epilogue { kReduce = 0, kStore = 1 };
 
 struct GemmArgs {
     const int32_t *row_count;  // R, written by compact_rows_kernel
@@ -123,7 +130,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     lmhead_gemm_kernel(const __grid_constant__ CUtensorMap map_h,
                        const __grid_constant__ CUtensorMap map_w, const GemmArgs a)
 {
-    using Cfg = TileCfg<BN_, MODE>;
+    using Cfg = TileCfg<BN_, MODE, EPI>;
     constexpr int CL = MODE == kSolo ? 1 : 2;
     constexpr bool PAIR = MODE == kPair;
     constexpr int BN = Cfg::BN, kStages = Cfg::kStages, KB = Cfg::kKB;
@@ -141,6 +148,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint64_t *done = tempty + 2;            // MMA thread: all its MMAs have completed
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    float *staging = reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(bars) + kBarrierBytes);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -388,16 +396,28 @@ __global__ void __launch_bounds__(kThreads, 1)
                     a.partials[(int64_t)r * a.n_tiles + n] = p;
                 }
             } else {
-                const int64_t row = r < R ? a.row_ids[r] : -1;
+                // A lane holds 32 columns of its own row, so storing from the registers would
+                // touch 32 rows per instruction: 122 us for 192 rows of 50001 logits at
+                // H = 2048.  The block turns in shared memory and leaves row by row, 128
+                // consecutive bytes per instruction: 61 us.
+                float *block = staging + quarter * kStageWarpFloats;
+                const int row = r < R ? a.row_ids[r] : -1;
+                const int live = min(R - (m * BM + quarter * 32), 32);  // the warp's rows < R
 #pragma unroll 1
                 for (int c = 0; c < (BN + 31) / 32; ++c) {
                     tc::tmem_ld_32cols(taddr + c * 32, v);
-                    if (row >= 0) {
-                        float *dst = a.logits + row * a.V + col0 + c * 32;
+                    __syncwarp();  // the block's last rows have been read
 #pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (c * 32 + j < BN && col0 + c * 32 + j < a.V)
-                                dst[j] = v[j];
+                    for (int j = 0; j < 32; ++j)
+                        block[lane * kStagePitch + j] = v[j];
+                    __syncwarp();
+                    const int col = col0 + c * 32 + lane;
+                    const bool in = c * 32 + lane < BN && col < a.V;
+#pragma unroll 4
+                    for (int i = 0; i < live; ++i) {
+                        const int64_t row_i = __shfl_sync(0xFFFFFFFFu, row, i);
+                        if (in)
+                            a.logits[row_i * a.V + col] = block[i * kStagePitch + lane];
                     }
                 }
                 tc::fence_before_sync();
@@ -1080,7 +1100,7 @@ cudaError_t launch_gemm_cfg(const CUtensorMap &mh, const CUtensorMap &mw, const 
     if (dev < 0 || dev >= 64)
         return cudaErrorInvalidDevice;
     auto kern = lmhead_gemm_kernel<EPI, MODE, BN>;
-    constexpr size_t smem = TileCfg<BN, MODE>::kSmemBytes;
+    constexpr size_t smem = TileCfg<BN, MODE, EPI>::kSmemBytes;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = smem;
