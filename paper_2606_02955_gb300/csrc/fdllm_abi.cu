@@ -121,22 +121,35 @@ fdllm_status owned_workspace(size_t need, cudaStream_t stream, void **out)
 
 namespace {
 
-// The layout of a call on the library-owned workspace, which grows to hold it.  It cannot grow
-// while `stream` is captured: what fits the workspace as it is serves there.
+size_t owned_bytes()
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
+        return 0;
+    std::lock_guard<std::mutex> lock(g_ws_mutex);
+    return g_ws[dev].bytes;
+}
+
+}  // namespace
+
+bool owned_workspace_ready(size_t need, cudaStream_t stream)
+{
+    if (need <= owned_bytes())
+        return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(stream, &cap) != cudaSuccess ||
+           cap == cudaStreamCaptureStatusNone;
+}
+
+namespace {
+
+// The layout of a call on the library-owned workspace, which grows to hold it except during a
+// capture: there what fits the workspace as it is serves.
 Layout owned_layout(int64_t rows, int64_t row_bytes, cudaStream_t stream)
 {
     const Layout l = layout_for(rows, row_bytes);
-    size_t have = 0;
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices) {
-        std::lock_guard<std::mutex> lock(g_ws_mutex);
-        have = g_ws[dev].bytes;
-    }
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (l.total <= have || cudaStreamIsCapturing(stream, &cap) != cudaSuccess ||
-        cap == cudaStreamCaptureStatusNone)
-        return l;
-    return layout_within(rows, row_bytes, have);
+    return owned_workspace_ready(l.total, stream) ? l
+                                                  : layout_within(rows, row_bytes, owned_bytes());
 }
 
 VocabReduceArgs reduce_args(const void *logits, int dtype, int B, int L, int V,

@@ -176,6 +176,10 @@ fdllm_status lmhead_select_owned(const void *hidden, const void *w_vocab, int B,
 // compact row count at 8.
 fdllm_status owned_workspace(size_t need, cudaStream_t stream, void **out);
 
+// Whether owned_workspace can give `need` bytes: the workspace holds them, or `stream` is not
+// being captured (the workspace cannot grow during a capture).
+bool owned_workspace_ready(size_t need, cudaStream_t stream);
+
 // fdllm_select's argument checks (shape, pointers, mode, param, logits alignment and the
 // unit plan's index range), done before anything is enqueued.
 fdllm_status check_select_args(const void *logits, int dtype, int B, int L, int V,

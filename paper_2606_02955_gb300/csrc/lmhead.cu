@@ -15,8 +15,10 @@
 //                            or CTA-pair (cta_group::2) variants
 //      lmhead_slab_kernel    (at most 32 rows) the operands swapped, W as the M = 128 side:
 //                            each CTA streams one vocabulary slab, one partial per row
+//      lmhead_wide_kernel    (up to 896 rows) the operands swapped on a CTA pair, W as the
+//                            M = 256 side and up to 256 (or 320) rows as N
 //   4. combine_rows_kernel   four warps per row fold its tile (or slab) partials in a fixed
-//                            order
+//      combine_wide_kernel   order; the wide variant's, laid out by tile, four rows per CTA
 //   5. profile_select        steps a2-a5 on the confidences (profile_select.cu)
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -55,6 +57,8 @@ enum Mode {
                      // rows and half of the W tile; the even CTA issues the MMAs for both
     kSlab = 3,       // at most 32 rows: W as the M = 128 operand, each CTA a vocabulary slab
                      // (lmhead_slab_kernel)
+    kWide = 4,       // W as the M = 256 operand of a CTA pair, the rows as its N
+                     // (lmhead_wide_kernel)
 };
 
 constexpr int PAIR_KB = 2;  // pair mode: K-blocks per stage
@@ -91,7 +95,9 @@ struct GemmArgs {
     int32_t k_blocks;          // ceil(H / BK)
     int32_t slab_tiles;        // slab variant: vocabulary tiles, ceil(V / slab_h)
     int32_t slab_h;            // slab variant: W rows per tile (a multiple of 8, <= 128)
-    UnitPartial *partials;     // kReduce: [R][n_tiles]
+    int32_t w_tiles;           // wide variant: vocabulary tiles of a CTA pair, ceil(V / kWideTile)
+    int32_t rows;              // wide variant: B * L, the row pitch of its partials
+    UnitPartial *partials;     // kReduce: [R][n_tiles]; wide variant: [n_tiles][rows]
     float *logits;             // kStore: [B * L][V] fp32, written at masked rows
     uint32_t *status;          // sticky device error bits
     bool pdl;                  // host side: launch as a programmatic dependent
@@ -116,6 +122,30 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, ui
                 return false;
             }
         }
+    }
+}
+
+// wait_or_abort by a converged warp, the same answer in every lane.
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, uint32_t *status,
+                                          volatile int *abort_flag)
+{
+    if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity)))
+        return true;
+    return __all_sync(0xFFFFFFFFu, wait_or_abort(bar, parity, status, abort_flag));
+}
+
+// Waits (bounded) for the last `filled` fills of a ring of `stages` stages whose next fill would
+// be that of stage s in phase ph: one thread, before its CTA may exit.
+__device__ __forceinline__ void drain_ring(uint64_t *full, int stages, int s, uint32_t ph,
+                                           uint32_t filled, uint32_t *status)
+{
+    for (uint32_t i = 0; i < filled; ++i) {
+        if (s == 0) {
+            s = stages;
+            ph ^= 1u;
+        }
+        --s;
+        mbar_wait(&full[s], ph, status, kDrainLimitNs);
     }
 }
 
@@ -727,6 +757,451 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
+// ----------------------------------------------------------------------------- wide variant
+// W is the M = 256 operand of a CTA pair (a tile of 256 vocabulary entries, 128 per CTA, lane =
+// entry) and the packed rows are N, in blocks of up to 256 rows (one MMA group, two accumulators
+// in turn) or, for 257 to 320 rows, one block of two groups that share every W stage (three
+// accumulators).  What bounds the solo variant at 2 to 6 row tiles is the 64 B/clock at which an
+// SM receives from L2: its stage is 42 KB for 416 MMA cycles (101 B/clock wanted, 65 measured).
+// Here a stage is (128 + N / 2) x 128 B for 2 N cycles: 75 B/clock at N = 192, 58 at 320, and no
+// row tile is padded to 128.  LLaDA's head, 3/4 of B x 32 rows, whole fdllm_lmhead_confidence
+// pass, this variant against the better of solo and pair: B = 3 (72 rows) 160 against 163 us,
+// 8 170 against 190, 12 204 against 251, 16 244 against 261, 24 346 against 396, 28 385 against
+// 410, 32 426 against 422 and 64 795 against 785 (pair): the host takes it up to 28 x 32 rows.
+// Other cuts measured: 288 rows in two blocks 220, 381 rows in one block of two groups 245, 480
+// rows in one block 311 against 293 in two.
+constexpr int kWideTile = 256;                  // vocabulary entries per CTA pair and item
+constexpr int kWideMaxGroup = 256;              // MMA columns per group
+constexpr int kWideTwoGroups = 320;             // rows that still make one block, of two groups
+constexpr int kWideMaxStages = 12;
+constexpr int kWideWarps = 12;                  // epilogue warps, three per TMEM lane quarter
+constexpr int kWideSplit = kWideWarps / 4;
+constexpr int kWideThreads = 64 + kWideWarps * 32;
+constexpr int kWideChunk = 8;                   // columns an epilogue warp turns at a time
+constexpr size_t kWideBarBytes = 512;
+constexpr int kWidePitch = kWideChunk + 1;      // both ways free of bank conflicts
+constexpr size_t kWideStaging = (size_t)kWideWarps * 32 * kWidePitch * 4;
+constexpr size_t kWideQuarters = (size_t)4 * kWideMaxGroup * (4 + 4 + 1);
+constexpr size_t kWideSmemBytes = 227 * 1024;
+constexpr size_t kWideFixed = kWideBarBytes + kWideStaging + kWideQuarters;
+static_assert((2 * kWideMaxStages + 2 * 4 + 1) * 8 + 8 <= (int)kWideBarBytes, "barriers");
+
+// Tensor maps of the packed rows, box heights 16, 32, ..., 128: entry h / 16 - 1 loads half a
+// group's rows.
+constexpr int kWideMaps = kWideMaxGroup / 32;
+struct WideRowMaps {
+    CUtensorMap m[kWideMaps];
+};
+
+// How R rows are cut: n_blocks blocks of `groups` groups of g rows each, g a multiple of 32 (what
+// lies past R is padding), items (W tile, block) with the block fastest, so that the pairs
+// sharing a W tile work on it at the same time.  `buffers` accumulators of g columns take turns.
+struct WideCut {
+    int n_blocks, groups, g, buffers;
+};
+
+__device__ __forceinline__ WideCut wide_cut(int R)
+{
+    WideCut c;
+    c.n_blocks = R > kWideTwoGroups ? (R + kWideMaxGroup - 1) / kWideMaxGroup : R > 0;
+    const int per = c.n_blocks > 0 ? (R + c.n_blocks - 1) / c.n_blocks : 1;
+    c.groups = per > kWideMaxGroup ? 2 : 1;
+    c.g = ((per + c.groups - 1) / c.groups + 31) / 32 * 32;
+    c.buffers = min(4, (int)kTmemCols / c.g);
+    return c;
+}
+
+// The items of one CTA pair.  Whole rounds of items over the pairs first; if what is left then
+// fills at most half of them and a block has two groups, each leftover item goes to two pairs,
+// one group each.
+struct WideItems {
+    int64_t whole, total;  // items of whole rounds, all items
+    int pairs, pair;
+    bool split;
+
+    __device__ __forceinline__ WideItems(const WideCut &c, int64_t n_w_tiles, int pairs_, int pair_)
+        : total(n_w_tiles * c.n_blocks), pairs(pairs_), pair(pair_)
+    {
+        const int64_t left = total % pairs;
+        whole = total - left;
+        split = c.groups == 2 && 2 * left <= pairs;
+    }
+    // The pair's i-th item: its index, or -1 past the last, and its groups [j0, j1).
+    __device__ __forceinline__ int64_t item(int64_t i, int groups, int &j0, int &j1) const
+    {
+        j0 = 0;
+        j1 = groups;
+        const int64_t t = i * pairs + pair;
+        if (t < whole)
+            return t;
+        if (i != whole / pairs)
+            return -1;
+        if (!split)
+            return t < total ? t : -1;
+        const int64_t u = whole + pair / 2;
+        j0 = pair & 1;
+        j1 = j0 + 1;
+        return u < total ? u : -1;
+    }
+};
+
+// bar.red over the epilogue warps: true when every thread's `ok` is true.
+__device__ __forceinline__ bool epilogue_all(bool ok)
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+                 "barrier.cta.red.and.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(r)
+                 : "r"((uint32_t)ok), "n"(kWideWarps * 32)
+                 : "memory");
+    return r != 0;
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(kWideThreads, 1)
+    lmhead_wide_kernel(const __grid_constant__ WideRowMaps maps_h,
+                       const __grid_constant__ CUtensorMap map_w, const GemmArgs a)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const uint32_t ring_bytes =
+        (uint32_t)(kWideSmemBytes - kWideFixed - (size_t)(smem - smem_raw)) / 1024 * 1024;
+    uint8_t *fixed = smem + ring_bytes;
+    uint64_t *full = reinterpret_cast<uint64_t *>(fixed);
+    uint64_t *empty = full + kWideMaxStages;
+    uint64_t *tfull = empty + kWideMaxStages;
+    uint64_t *tempty = tfull + 4;
+    uint64_t *done = tempty + 4;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    float *staging = reinterpret_cast<float *>(fixed + kWideBarBytes);
+    float *q_M = reinterpret_cast<float *>(fixed + kWideBarBytes + kWideStaging);  // [4][256]
+    float *q_S = q_M + 4 * kWideMaxGroup;
+    uint8_t *q_I = reinterpret_cast<uint8_t *>(q_S + 4 * kWideMaxGroup);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kWideMaxStages; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int i = 0; i < 4; ++i) {
+            mbar_init(&tfull[i], 1);
+            mbar_init(&tempty[i], 2 * kWideWarps);
+        }
+        mbar_init(done, 1);
+        *abort_flag = 0;
+        fence_mbar_init();
+        tc::prefetch_tensormap(&map_w);
+    }
+    if (warp == 1)
+        tc::tmem_alloc_pair(tmem_slot, kTmemCols);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::cluster_sync();  // the peer's barriers are initialised before any remote signal
+    tc::fence_after_sync();
+    const uint32_t tmem_base = *tmem_slot;
+
+    pdl_wait();  // the packed rows and their count are complete
+
+    const int rank = (int)tc::cluster_ctarank();
+    const int R = __shfl_sync(0xFFFFFFFFu, *a.row_count, 0);
+    const WideCut cut = wide_cut(R);
+    const int block_rows = cut.groups * cut.g;
+    const uint32_t half_bytes = (uint32_t)(cut.g / 2 * BK * 2);  // a CTA's share of a group's stage
+    const uint32_t stage_bytes = kABytes + cut.groups * half_bytes;
+    const int stages = min(kWideMaxStages, (int)(ring_bytes / stage_bytes));
+    const WideItems items(cut, a.w_tiles, (int)tc::cluster_count_x(), (int)tc::cluster_id_x());
+
+    // Warps 0 and 1 run whole, one elected lane issuing: loop state and operand addresses then
+    // stay warp-uniform, which the issuing instructions need them to be.
+    if (warp == 0) {
+        const uint64_t pol = make_evict_first_policy();  // W is read once (per row block)
+        const CUtensorMap *map_h = &maps_h.m[cut.g / 32 - 1];
+        int s = 0;
+        uint32_t ph = 0, filled = 0;
+        bool ok = true;
+        int j0, j1;
+        for (int64_t i = 0; ok; ++i) {
+            const int64_t t = items.item(i, cut.groups, j0, j1);
+            if (t < 0)
+                break;
+            const int n = (int)(t / cut.n_blocks);
+            const int row0 = (int)(t % cut.n_blocks) * block_rows + rank * (cut.g / 2);
+            const int w_row = n * kWideTile + rank * BM;
+            const uint32_t bytes = kABytes + (uint32_t)(j1 - j0) * half_bytes;
+            for (int kb = 0; kb < a.k_blocks; ++kb) {
+                if (!warp_wait(&empty[s], ph ^ 1u, a.status, abort_flag)) {
+                    ok = false;
+                    break;
+                }
+                if (elect_one()) {
+                    // Both CTAs' bytes complete on the even CTA's barrier, which it arms.
+                    if (rank == 0)
+                        mbar_arrive_expect_tx(&full[s], 2 * bytes);
+                    const uint32_t bar0 = tc::map_to_rank(&full[s], 0);
+                    uint8_t *stage = smem + s * stage_bytes;
+                    tc::tma_load_2d_pair_hint(stage, &map_w, kb * BK, w_row, bar0, pol);
+                    tc::tma_load_2d_pair(stage + kABytes, map_h, kb * BK, row0 + j0 * cut.g, bar0);
+                    if (j1 - j0 == 2)
+                        tc::tma_load_2d_pair(stage + kABytes + half_bytes, map_h, kb * BK,
+                                             row0 + cut.g, bar0);
+                }
+                filled = min(filled + 1, (uint32_t)stages);
+                if (++s == stages) {
+                    s = 0;
+                    ph ^= 1u;
+                }
+            }
+        }
+        // No copy may still be in flight when the pair exits (the odd CTA leaves only after
+        // the even one, at the final cluster barrier): the last fill of each stage.
+        if (rank == 0 && elect_one())
+            drain_ring(full, stages, s, ph, filled, a.status);
+        __syncwarp();
+    } else if (warp == 1) {
+        if (rank == 0) {
+            const uint32_t idesc = tc::idesc_bf16_f32(2 * BM, cut.g);
+            int s = 0;
+            uint32_t ph = 0;
+            uint32_t used = 0;  // groups accumulated so far
+            bool ok = true;
+            int j0, j1;
+            for (int64_t i = 0; ok; ++i) {
+                const int64_t t = items.item(i, cut.groups, j0, j1);
+                if (t < 0)
+                    break;
+                const bool two = j1 - j0 == 2;
+                const uint32_t b0 = used % cut.buffers, b1 = (used + 1) % cut.buffers;
+                const uint32_t turn1 = (used + 1) / cut.buffers;
+                if (!warp_wait(&tempty[b0], (used / cut.buffers & 1u) ^ 1u, a.status, abort_flag))
+                    break;
+                tc::fence_after_sync();
+                const uint32_t d0 = tmem_base + b0 * cut.g, d1 = tmem_base + b1 * cut.g;
+                // Two groups share each stage.  While the second group's accumulator is still
+                // being read, the first one runs ahead over the stages of the ring (k0, at s);
+                // the second one follows (k1, at s1), the last to read a stage.
+                bool free1 = !two;
+                int k0 = 0, k1 = 0, s1 = s;
+                while (k1 < a.k_blocks) {
+                    if (k0 == k1 || (!free1 && k0 < a.k_blocks && k0 - k1 < stages)) {
+                        if (!warp_wait(&full[s], ph, a.status, abort_flag)) {
+                            ok = false;
+                            break;
+                        }
+                        tc::fence_after_sync();
+                        const uint64_t ad = tc::sw128_kmajor_desc(smem + s * stage_bytes);
+                        const uint64_t bd = ad + (kABytes >> 4);
+                        if (elect_one()) {
+#pragma unroll
+                            for (int k = 0; k < BK / 16; ++k)
+                                tc::mma_bf16_pair(d0, ad + 2u * k, bd + 2u * k, idesc,
+                                                  (k0 | k) != 0);
+                            if (!two)
+                                tc::commit_pair_multicast(&empty[s]);
+                            if (k0 == a.k_blocks - 1)
+                                tc::commit_pair_multicast(&tfull[b0]);
+                        }
+                        ++k0;
+                        if (++s == stages) {
+                            s = 0;
+                            ph ^= 1u;
+                        }
+                        if (!two) {
+                            ++k1;
+                            continue;
+                        }
+                        if (!free1) {
+                            free1 = __all_sync(0xFFFFFFFFu,
+                                               mbar_try_wait(&tempty[b1], (turn1 & 1u) ^ 1u));
+                            if (!free1 && k0 < a.k_blocks && k0 - k1 < stages)
+                                continue;
+                            if (!free1 && !warp_wait(&tempty[b1], (turn1 & 1u) ^ 1u, a.status,
+                                                     abort_flag)) {
+                                ok = false;
+                                break;
+                            }
+                            free1 = true;
+                            tc::fence_after_sync();
+                        }
+                    }
+                    const uint64_t ad = tc::sw128_kmajor_desc(smem + s1 * stage_bytes);
+                    const uint64_t bd = ad + (kABytes >> 4) + (half_bytes >> 4);
+                    if (elect_one()) {
+#pragma unroll
+                        for (int k = 0; k < BK / 16; ++k)
+                            tc::mma_bf16_pair(d1, ad + 2u * k, bd + 2u * k, idesc, (k1 | k) != 0);
+                        tc::commit_pair_multicast(&empty[s1]);
+                    }
+                    ++k1;
+                    if (++s1 == stages)
+                        s1 = 0;
+                }
+                if (!ok)
+                    break;
+                if (two && elect_one())
+                    tc::commit_pair_multicast(&tfull[b1]);
+                const int ng = j1 - j0;
+                used += ng;
+            }
+            // Tensor memory is freed below only after every MMA issued here has completed.
+            __syncwarp();
+            if (elect_one()) {
+                tc::commit_pair_multicast(done);  // the odd CTA's copy is never waited on
+                mbar_wait(done, 0, a.status, kDrainLimitNs);
+            }
+        }
+        __syncwarp();
+    } else {
+        // Epilogue: warp w reads TMEM lanes [32 (w % 4), +32) and every third chunk of 8
+        // columns, all of a group's into registers first, which hands the accumulator back after
+        // a few hundred cycles.  A lane's columns are rows of one vocabulary entry, so each 32 x 8
+        // block turns in shared memory: lane l then holds entries 8 (l / 8) + 0..7 of column
+        // l % 8.
+        const int quarter = warp & 3, parity = (warp - 2) >> 2;
+        const int et = threadIdx.x - 64;
+        float *block = staging + (warp - 2) * 32 * kWidePitch;
+        const int col = lane & 7, e0 = lane & ~7;
+        uint32_t used = 0;
+        int j0, j1;
+        bool ok = true;
+        for (int64_t i = 0; ok; ++i) {
+            const int64_t t = items.item(i, cut.groups, j0, j1);
+            if (t < 0)
+                break;
+            const int n = (int)(t / cut.n_blocks);
+            const int blk0 = (int)(t % cut.n_blocks) * block_rows;
+            const int ent0 = n * kWideTile + rank * BM;
+            const int ent = ent0 + quarter * 32 + lane;
+            for (int j = j0; j < j1; ++j, ++used) {
+                const uint32_t buf = used % cut.buffers, turn = used / cut.buffers;
+                const bool got = wait_or_abort(&tfull[buf], turn & 1u, a.status, abort_flag);
+                // All epilogue warps go on or leave together (they share barriers below); past
+                // this one the last group's quarter results have been read.
+                if (!epilogue_all(got)) {
+                    ok = false;
+                    break;
+                }
+                tc::fence_after_sync();
+                const uint32_t taddr =
+                    tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * cut.g;
+                const int row0 = blk0 + j * cut.g;
+                const int live = min(cut.g, R - row0);  // columns that are rows
+                // Eight chunks (192 of the group's columns) per pass fit the registers.
+                constexpr int kChunks = 8, kPassCols = kChunks * kWideSplit * kWideChunk;
+#pragma unroll 1
+                for (int p0 = 0; p0 < cut.g; p0 += kPassCols) {
+                    float x[kChunks][kWideChunk];
+#pragma unroll
+                    for (int q = 0; q < kChunks; ++q)
+                        if (p0 + (kWideSplit * q + parity) * kWideChunk < live)
+                            tc::tmem_ld_8cols_async(
+                                taddr + p0 + (kWideSplit * q + parity) * kWideChunk, x[q]);
+                    tc::tmem_wait_ld();
+#pragma unroll
+                    for (int q = 0; q < kChunks; ++q)
+                        tc::tie_regs(x[q]);
+                    if (p0 + kPassCols >= cut.g) {  // the accumulator has been read
+                        tc::fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) {
+                            if (rank != 0)
+                                tc::mbar_arrive_remote(tc::map_to_rank(&tempty[buf], 0));
+                            else
+                                mbar_arrive(&tempty[buf]);
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < kChunks; ++q) {
+                        const int c = p0 + (kWideSplit * q + parity) * kWideChunk;
+                        if (c >= live)
+                            break;
+                        float(&v)[kWideChunk] = x[q];
+                        if (EPI == kStore) {
+                            const int mine = c + col < live ? a.row_ids[row0 + c + col] : 0;
+#pragma unroll
+                            for (int k = 0; k < kWideChunk; ++k) {
+                                const int64_t row = __shfl_sync(0xFFFFFFFFu, mine, k);
+                                if (c + k < live && ent < a.V)
+                                    a.logits[row * a.V + ent] = v[k];
+                            }
+                            continue;
+                        }
+                        if (ent >= a.V)  // past the vocabulary (the last tile's zero-filled W rows)
+#pragma unroll
+                            for (int k = 0; k < kWideChunk; ++k)
+                                v[k] = -INFINITY;
+                        __syncwarp();  // the block's previous columns have been read
+#pragma unroll
+                        for (int k = 0; k < kWideChunk; ++k)
+                            block[lane * kWidePitch + k] = v[k];
+                        __syncwarp();
+                        float M = -INFINITY;
+#pragma unroll
+                        for (int k = 0; k < kWideChunk; ++k) {
+                            v[k] = block[(e0 + k) * kWidePitch + col];
+                            M = fmaxf(M, v[k]);
+                        }
+                        M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, 8));
+                        M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, 16));
+                        // exp(x - M) as (x - M) * log2e, exact at any magnitude; NaN poisons S, -inf
+                        // adds nothing
+                        const float base = M == -INFINITY ? 0.0f : M;
+                        float S2[2] = {0.0f, 0.0f};
+                        int first = 255;
+#pragma unroll
+                        for (int k = kWideChunk - 1; k >= 0; --k) {
+                            first = v[k] == M ? e0 + k : first;
+                            S2[k & 1] += ex2_mufu((v[k] - base) * kLog2e);
+                        }
+                        float S = S2[0] + S2[1];
+                        S += __shfl_xor_sync(0xFFFFFFFFu, S, 8);
+                        S += __shfl_xor_sync(0xFFFFFFFFu, S, 16);
+                        first = min(first, __shfl_xor_sync(0xFFFFFFFFu, first, 8));
+                        first = min(first, __shfl_xor_sync(0xFFFFFFFFu, first, 16));
+                        if (e0 == 0) {
+                            q_M[quarter * kWideMaxGroup + c + col] = M;
+                            q_S[quarter * kWideMaxGroup + c + col] = S;
+                            q_I[quarter * kWideMaxGroup + c + col] = (uint8_t)first;
+                        }
+                    }
+                }
+                if (EPI == kReduce) {
+                    asm volatile("barrier.cta.sync 2, %0;" ::"n"(kWideWarps * 32) : "memory");
+                    if (et < live) {  // one row's four quarters, in entry order
+                        float M = -INFINITY, S = 0.0f;
+                        uint32_t I = kNoIdx;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const uint32_t e = q_I[q * kWideMaxGroup + et];
+                            fold_state(M, S, I, q_M[q * kWideMaxGroup + et],
+                                       q_S[q * kWideMaxGroup + et],
+                                       e < 32 ? (uint32_t)(ent0 + q * 32) + e : kNoIdx);
+                        }
+                        UnitPartial p;
+                        p.M = S != S ? __int_as_float(0x7FC00000) : M;
+                        p.S = M == -INFINITY ? 0.0f : S;
+                        p.idx = I;
+                        p.pad = 0;
+                        a.partials[(int64_t)(2 * n + rank) * a.rows + row0 + et] = p;
+                    }
+                }
+            }
+        }
+    }
+    if (threadIdx.x == 0)
+        pdl_launch_dependents();  // the row combination may start launching
+    __syncthreads();
+    tc::cluster_sync();  // both CTAs are done with the pair's tensor memory
+    if (warp == 1) {
+        __syncwarp();
+        tc::fence_after_sync();
+        tc::tmem_dealloc_pair(tmem_base, kTmemCols);
+    }
+    tc::cluster_sync();  // no CTA leaves while its peer may still write into it
+}
+
 // One CTA: the packed list of masked rows (ascending) and its length.
 __global__ void __launch_bounds__(1024) compact_rows_kernel(const uint8_t *mask, int rows,
                                                             int32_t *row_ids, int32_t *row_count)
@@ -810,6 +1285,34 @@ __device__ __forceinline__ Part fold(const Part &x, const Part &y)
     return r;
 }
 
+__device__ __forceinline__ Part as_part(const int4 &v)
+{
+    Part y{__int_as_float(v.x), __int_as_float(v.y), (uint32_t)v.z, false};
+    y.nan = y.M != y.M;
+    if (y.nan)
+        y.M = -__int_as_float(0x7F800000);
+    return y;
+}
+
+__device__ __forceinline__ Part shfl_part(const Part &x, int o)
+{
+    Part y;
+    y.M = __shfl_xor_sync(0xFFFFFFFFu, x.M, o);
+    y.S = __shfl_xor_sync(0xFFFFFFFFu, x.S, o);
+    y.idx = __shfl_xor_sync(0xFFFFFFFFu, x.idx, o);
+    y.nan = __shfl_xor_sync(0xFFFFFFFFu, (int)x.nan, o) != 0;
+    return y;
+}
+
+// c = min(1/S, 1) and x_hat of a whole row; NaN and -1 with a NaN logit or an infinite maximum.
+__device__ __forceinline__ void store_conf(const Part &x, int row, float *conf, int32_t *tok)
+{
+    const bool finite = fabsf(x.M) <= 3.402823466e38f && fabsf(x.S) <= 3.402823466e38f;
+    const bool bad = x.nan || !finite || !(x.S > 0.0f) || x.idx == kNoIdx;
+    conf[row] = bad ? __int_as_float(0x7FC00000) : fminf(1.0f / x.S, 1.0f);
+    tok[row] = bad ? -1 : (int32_t)x.idx;
+}
+
 // One CTA of kCombineWarps warps per packed row: lane l of warp q folds tiles
 // q * 32 + l + 128 i (i = 0, 1, ...) in order, the lanes of each warp fold in a fixed
 // butterfly, and the warps' results fold in warp order.  A fixed tree, so the result does not
@@ -841,23 +1344,12 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
                 v[b] = __ldcg(reinterpret_cast<const int4 *>(p + j0 + kStride * b));
 #pragma unroll
         for (int b = 0; b < kBatch; ++b)
-            if (j0 + kStride * b < n_tiles) {
-                Part y{__int_as_float(v[b].x), __int_as_float(v[b].y), (uint32_t)v[b].z, false};
-                y.nan = y.M != y.M;
-                if (y.nan)
-                    y.M = -__int_as_float(0x7F800000);
-                acc = fold(acc, y);
-            }
+            if (j0 + kStride * b < n_tiles)
+                acc = fold(acc, as_part(v[b]));
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        Part y;
-        y.M = __shfl_xor_sync(0xFFFFFFFFu, acc.M, o);
-        y.S = __shfl_xor_sync(0xFFFFFFFFu, acc.S, o);
-        y.idx = __shfl_xor_sync(0xFFFFFFFFu, acc.idx, o);
-        y.nan = __shfl_xor_sync(0xFFFFFFFFu, (int)acc.nan, o) != 0;
-        acc = fold(acc, y);
-    }
+    for (int o = 16; o > 0; o >>= 1)
+        acc = fold(acc, shfl_part(acc, o));
     if (lane == 0)
         s_part[q] = acc;
     __syncthreads();
@@ -865,15 +1357,56 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
         acc = s_part[0];
         for (int w = 1; w < kCombineWarps; ++w)
             acc = fold(acc, s_part[w]);
-        const int row = row_ids[r];
-        const bool finite = fabsf(acc.M) <= 3.402823466e38f && fabsf(acc.S) <= 3.402823466e38f;
-        if (acc.nan || !finite || !(acc.S > 0.0f) || acc.idx == kNoIdx) {
-            conf[row] = __int_as_float(0x7FC00000);
-            tok[row] = -1;
-        } else {
-            conf[row] = fminf(1.0f / acc.S, 1.0f);
-            tok[row] = (int32_t)acc.idx;
+        store_conf(acc, row_ids[r], conf, tok);
+    }
+}
+
+// The wide variant's partials [n_tiles][rows]: a CTA takes kWideRows neighbouring rows (one
+// 64-byte segment per tile), thread t row t % 4 and tiles t / 4, t / 4 + 64, ... in order, then
+// the same symmetric folds: three butterfly steps per warp, the warps in order.
+constexpr int kWideRows = 4;
+constexpr int kWideFoldThreads = 256;
+
+__global__ void __launch_bounds__(kWideFoldThreads)
+    combine_wide_kernel(const UnitPartial *partials, int n_tiles, int rows, const int32_t *row_ids,
+                        const int32_t *row_count, float *conf, int32_t *tok)
+{
+    constexpr int kTileLanes = kWideFoldThreads / kWideRows;
+    __shared__ Part s_part[kWideFoldThreads / 32][kWideRows];
+    pdl_wait();  // every tile partial is written
+    if (threadIdx.x == 0)
+        pdl_launch_dependents();
+    const int R = *row_count;
+    const int r = blockIdx.x * kWideRows + threadIdx.x % kWideRows;
+    if (blockIdx.x * kWideRows >= R)
+        return;
+    Part acc{-__int_as_float(0x7F800000), 0.0f, kNoIdx, false};
+    constexpr int kBatch = 8;  // loads in flight per thread before the folds
+    if (r < R)
+        for (int t0 = threadIdx.x / kWideRows; t0 < n_tiles; t0 += kTileLanes * kBatch) {
+            int4 v[kBatch];
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b)
+                if (t0 + kTileLanes * b < n_tiles)
+                    v[b] = __ldcg(reinterpret_cast<const int4 *>(
+                        partials + (int64_t)(t0 + kTileLanes * b) * rows + r));
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b)
+                if (t0 + kTileLanes * b < n_tiles)
+                    acc = fold(acc, as_part(v[b]));
         }
+#pragma unroll
+    for (int o = 16; o >= kWideRows; o >>= 1)
+        acc = fold(acc, shfl_part(acc, o));
+    const int lane = threadIdx.x & 31;
+    if (lane < kWideRows)
+        s_part[threadIdx.x >> 5][lane] = acc;
+    __syncthreads();
+    if (threadIdx.x < kWideRows && r < R) {
+        acc = s_part[0][lane];
+        for (int w = 1; w < kWideFoldThreads / 32; ++w)
+            acc = fold(acc, s_part[w][lane]);
+        store_conf(acc, row_ids[r], conf, tok);
     }
 }
 
@@ -1023,11 +1556,11 @@ bool slab_preferred(int V)
     return slab_rows <= tile_rows;
 }
 
-// The GEMM variant: for at most kSlabRows rows the slab variant where slab_preferred; else
-// kPair (cta_group::2) when at least 8 row tiles can share every W tile, kSolo below that
-// (the pair pads to an even number of row tiles, and W streaming from HBM, not
-// shared-memory bandwidth, is the limit there).  FDLLM_LMHEAD_GEMM = solo, pair or slab
-// forces one (slab only where B * L <= kSlabRows).
+// The GEMM variant: for at most kSlabRows rows the slab variant where slab_preferred, up to
+// kWideRowsMax rows the wide one, the pair beyond (both sides measured at lmhead_wide_kernel).
+// FDLLM_LMHEAD_GEMM = solo, pair, slab or wide forces one (slab only where B * L <= kSlabRows).
+constexpr int kWideRowsMax = 28 * 32;
+
 int gemm_mode(int64_t rows, int V)
 {
     if (const char *e = std::getenv("FDLLM_LMHEAD_GEMM")) {
@@ -1038,10 +1571,12 @@ int gemm_mode(int64_t rows, int V)
             return kPair;
         if (v == "slab" && rows <= kSlabRows)
             return kSlab;
+        if (v == "wide")
+            return kWide;
     }
     if (rows <= kSlabRows && slab_preferred(V))
         return kSlab;
-    return (rows + BM - 1) / BM >= 8 ? kPair : kSolo;
+    return rows <= kWideRowsMax ? kWide : kPair;
 }
 
 int sm_count()
@@ -1167,6 +1702,48 @@ cudaError_t launch_slab(const CUtensorMap &mh, const CUtensorMap &mw, const Gemm
 }
 
 template <int EPI>
+cudaError_t launch_wide(const WideRowMaps &mh, const CUtensorMap &mw, const GemmArgs &g,
+                        cudaStream_t stream)
+{
+    static std::once_flag once[64];
+    static int grid[64];
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess)
+        return err;
+    if (dev < 0 || dev >= 64)
+        return cudaErrorInvalidDevice;
+    auto kern = lmhead_wide_kernel<EPI>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kWideThreads);
+    cfg.dynamicSmemBytes = kWideSmemBytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;  // the occupancy query below sees the cluster shape only
+    std::call_once(once[dev], [&] {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kWideSmemBytes);
+        const int sms = sm_count();
+        int clusters = 0;
+        cfg.gridDim = dim3((unsigned)(sms / 2 * 2));
+        if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1)
+            clusters = sms / 2;
+        (void)cudaGetLastError();
+        grid[dev] = clusters * 2;  // persistent: every pair resident at once
+    });
+    cfg.gridDim = dim3((unsigned)grid[dev]);
+    cfg.numAttrs = g.pdl ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, mh, mw, g);
+}
+
+template <int EPI>
 cudaError_t launch_gemm(const CUtensorMap &mh, const CUtensorMap &mw, const GemmArgs &g,
                         int mode, int bn, cudaStream_t stream)
 {
@@ -1184,11 +1761,28 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
                         uint8_t **ws_out, LmLayout *lay_out, bool pdl = true)
 {
     const int64_t rows = (int64_t)B * L;
-    const int mode = gemm_mode(rows, V);
-    const int bn = mode == kSlab ? slab_height(V) : choose_bn(rows, V, mode == kPair);
-    // partials per row: one per vocabulary tile, or one per CTA of the slab variant
-    const int n_tiles = mode == kSlab ? slab_grid(V) : (V + bn - 1) / bn;
-    const LmLayout lay = lm_layout(rows, H, n_tiles);
+    int mode = gemm_mode(rows, V);
+    int bn = 0, n_tiles = 0;
+    const int w_tiles = (V + kWideTile - 1) / kWideTile;
+    LmLayout lay;
+    // partials per row: one per vocabulary tile (per CTA of the pair in the wide variant), or
+    // one per CTA of the slab variant
+    auto plan = [&] {
+        bn = mode == kSlab   ? slab_height(V)
+             : mode == kWide ? kWideTile / 2
+                             : choose_bn(rows, V, mode == kPair);
+        n_tiles = mode == kSlab   ? slab_grid(V)
+                  : mode == kWide ? 2 * w_tiles
+                                  : (V + bn - 1) / bn;
+        lay = lm_layout(rows, H, n_tiles);
+    };
+    plan();
+    // Under capture the workspace cannot grow; one left by larger calls of the tile variants,
+    // whose partials are fewer, may hold only those.
+    if (mode == kWide && !owned_workspace_ready(lay.total, s)) {
+        mode = (rows + BM - 1) / BM >= 8 ? kPair : kSolo;
+        plan();
+    }
     void *wsv = nullptr;
     fdllm_status st = owned_workspace(lay.total, s, &wsv);
     if (st != FDLLM_OK)
@@ -1199,9 +1793,16 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
     uint8_t *packed = ws + lay.packed;
 
     CUtensorMap mh, mw;
-    if (!make_map(&mh, packed, H, rows, mode == kSlab ? kSlabRows : BM) ||
-        !make_map(&mw, w, H, V, mode == kSolo || mode == kSlab ? bn : bn / 2))
+    WideRowMaps wide_maps;
+    if (!make_map(&mw, w, H, V, mode == kPair ? bn / 2 : bn))
         return FDLLM_ERR_CUDA;
+    if (mode == kWide) {
+        for (int i = 0; i < kWideMaps && 32 * i < rows; ++i)  // groups no wider than the rows
+            if (!make_map(&wide_maps.m[i], packed, H, rows, 16 * (i + 1)))
+                return FDLLM_ERR_CUDA;
+    } else if (!make_map(&mh, packed, H, rows, mode == kSlab ? kSlabRows : BM)) {
+        return FDLLM_ERR_CUDA;
+    }
 
     if (launch_pdl(pdl, compact_rows_kernel, 1, 1024, s, mask, (int)rows, row_ids, row_count) !=
             cudaSuccess ||
@@ -1218,15 +1819,29 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
     g.k_blocks = (H + BK - 1) / BK;
     g.slab_h = mode == kSlab ? bn : 0;
     g.slab_tiles = mode == kSlab ? (V + bn - 1) / bn : 0;
+    g.w_tiles = w_tiles;
+    g.rows = (int)rows;
     g.partials = reinterpret_cast<UnitPartial *>(ws + lay.partials);
     g.logits = out_logits;
     g.status = reinterpret_cast<uint32_t *>(ws);
     g.pdl = pdl;
-    const cudaError_t e = epi == kReduce ? launch_gemm<kReduce>(mh, mw, g, mode, bn, s)
-                                         : launch_gemm<kStore>(mh, mw, g, mode, bn, s);
+    cudaError_t e;
+    if (mode == kWide)
+        e = epi == kReduce ? launch_wide<kReduce>(wide_maps, mw, g, s)
+                           : launch_wide<kStore>(wide_maps, mw, g, s);
+    else
+        e = epi == kReduce ? launch_gemm<kReduce>(mh, mw, g, mode, bn, s)
+                           : launch_gemm<kStore>(mh, mw, g, mode, bn, s);
     if (e != cudaSuccess)
         return FDLLM_ERR_CUDA;
-    if (epi == kReduce) {
+    if (epi == kReduce && mode == kWide) {
+        if (launch_pdl(pdl, combine_wide_kernel, (unsigned)((rows + kWideRows - 1) / kWideRows),
+                       kWideFoldThreads, s, (const UnitPartial *)g.partials, n_tiles, (int)rows,
+                       (const int32_t *)row_ids, (const int32_t *)row_count,
+                       reinterpret_cast<float *>(ws + lay.conf),
+                       reinterpret_cast<int32_t *>(ws + lay.tok)) != cudaSuccess)
+            return FDLLM_ERR_CUDA;
+    } else if (epi == kReduce) {
         if (launch_pdl(pdl, combine_rows_kernel, (unsigned)rows, kCombineWarps * 32,
                        s, (const UnitPartial *)g.partials, n_tiles, (const int32_t *)row_ids,
                        (const int32_t *)row_count, reinterpret_cast<float *>(ws + lay.conf),

@@ -29,6 +29,16 @@ __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
                  : "memory");
 }
 
+// True in exactly one lane of a converged warp.  A branch on it, unlike one on the lane index,
+// tells the compiler that a single thread runs what follows.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(r));
+    return r != 0;
+}
+
 // Makes barrier initialisation visible to the async (TMA) proxy and the rest of the CTA.
 __device__ __forceinline__ void fence_mbar_init()
 {
