@@ -61,13 +61,13 @@ enum Mode {
                      // (lmhead_wide_kernel)
 };
 
-constexpr int PAIR_KB = 2;  // pair mode: K-blocks per stage
-
 // Vocabulary entries per tile (the MMA's N and the fp32 accumulator's width): 256, or 208,
 // which splits LLaDA's V = 126464 into 608 = 4 x 152 tiles, whole waves over 152 SMs.  The
-// stage count fills the ring budget: solo 4 x 48 KB at 256, 5 x 42 KB at 208; pair 3 x 64 KB
-// at 256 (each CTA holds half the W tile, and a stage two K-blocks: with the pair's two
-// cross-CTA signals per stage, fewer and larger stages measured faster than 6 x 32 KB).
+// stage count fills the ring budget: solo 4 x 48 KB at 256, 5 x 42 KB at 208; pair 6 x 32 KB
+// at 256 (each CTA holds half the W tile).  Three pair stages of two K-blocks each were the
+// faster ring while issuing a stage cost as much as its MMAs; with warp-uniform issue the finer
+// ring is: 28 x 32 rows 410 against 431 us, 32 x 32 rows 422 against 425, 64 x 32 rows 785
+// against 787.
 enum Epilogue { kReduce = 0, kStore = 1 };
 
 template <int BN_, int MODE, int EPI = kReduce>
@@ -75,8 +75,7 @@ struct TileCfg {
     static constexpr int BN = BN_;
     static constexpr int kBRows = MODE == kPair ? BN / 2 : BN;  // W rows held per CTA
     static constexpr int kBBytes = kBRows * BK * 2;
-    static constexpr int kKB = MODE == kPair ? PAIR_KB : 1;       // K-blocks of BK per stage
-    static constexpr int kStageBytes = kKB * (kABytes + kBBytes);
+    static constexpr int kStageBytes = kABytes + kBBytes;
     static constexpr size_t kStagingBytes = EPI == kStore ? 4 * kStageWarpFloats * 4 : 0;
     static constexpr int kFit = (int)((kRingBudget - kStagingBytes) / kStageBytes);
     static constexpr int kStages = kFit > 8 ? 8 : kFit;
@@ -163,14 +162,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     using Cfg = TileCfg<BN_, MODE, EPI>;
     constexpr int CL = MODE == kSolo ? 1 : 2;
     constexpr bool PAIR = MODE == kPair;
-    constexpr int BN = Cfg::BN, kStages = Cfg::kStages, KB = Cfg::kKB;
+    constexpr int BN = Cfg::BN, kStages = Cfg::kStages;
     constexpr int kBBytes = Cfg::kBBytes, kStageBytes = Cfg::kStageBytes;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t *sA = smem;                          // kStages x KB x [BM rows][128 B], swizzled
-    uint8_t *sB = smem + kStages * KB * kABytes; // kStages x KB x [kBRows rows][128 B]
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sB + kStages * KB * kBBytes);
+    uint8_t *sA = smem;                      // kStages x [BM rows][128 B], swizzled
+    uint8_t *sB = smem + kStages * kABytes;  // kStages x [kBRows rows][128 B]
+    uint64_t *bars = reinterpret_cast<uint64_t *>(sB + kStages * kBBytes);
     uint64_t *full = bars;                  // TMA -> MMA, one per stage
     uint64_t *empty = bars + kStages;       // MMA -> TMA, one per stage
     uint64_t *tfull = bars + 2 * kStages;   // MMA -> epilogue, one per accumulator
@@ -224,7 +223,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         else
             mbar_arrive(bar);
     };
-    const int R = *a.row_count;
+    const int R = __shfl_sync(0xFFFFFFFFu, *a.row_count, 0);
     const int num_m = (R + BM - 1) / BM;
     const int num_mc = (num_m + CL - 1) / CL;  // row-tile groups, one per cluster
     const int64_t total = (int64_t)num_mc * a.n_tiles;
@@ -234,67 +233,55 @@ __global__ void __launch_bounds__(kThreads, 1)
     // an odd number of row tiles, the last rank-1 CTA computes a tile of rows >= R (zero or
     // stale inputs) that its epilogue skips.
 
+    // Warps 0 and 1 run whole, one elected lane issuing: loop state and operand addresses then
+    // stay warp-uniform, which the issuing instructions need them to be.  Against loops under
+    // `lane == 0` (and the pair's stages as they were): 32 x 32 rows 434 against 439 us, 64 x 32
+    // 800 against 807, the slab variant at 24 rows 154.3 against 156.8.
     if (warp == 0) {
-        if (lane == 0) {
-            // W tiles are marked first to evict: each is read from HBM once, and the other row
-            // tiles that share it (consecutive work items) read it from L2 right away.
-            const uint64_t pol = make_evict_first_policy();
-            int s = 0;
-            uint32_t ph = 0;
-            uint32_t last_ph[kStages];
-            bool used[kStages];
-            for (int i = 0; i < kStages; ++i)
-                used[i] = false;
-            bool ok = true;
-            for (int64_t t = first; ok && t < total; t += stride) {
-                const int m = (int)(t % num_mc) * CL + rank, n = (int)(t / num_mc);
-                for (int kb = 0; kb < a.k_blocks; kb += KB) {
-                    if (!wait_or_abort(&empty[s], ph ^ 1u, a.status, abort_flag)) {
-                        ok = false;
-                        break;
-                    }
+        // W tiles are marked first to evict: each is read from HBM once, and the other row
+        // tiles that share it (consecutive work items) read it from L2 right away.
+        const uint64_t pol = make_evict_first_policy();
+        int s = 0;
+        uint32_t ph = 0, filled = 0;
+        bool ok = true;
+        for (int64_t t = first; ok && t < total; t += stride) {
+            const int m = (int)(t % num_mc) * CL + rank, n = (int)(t / num_mc);
+            for (int kb = 0; kb < a.k_blocks; ++kb) {
+                if (!warp_wait(&empty[s], ph ^ 1u, a.status, abort_flag)) {
+                    ok = false;
+                    break;
+                }
+                if (elect_one()) {
                     if constexpr (PAIR) {
-                        // Both CTAs' bytes complete on the even CTA's barrier, which it arms
-                        // (K-blocks past H, in the last stage when k_blocks is odd, are
-                        // zero-filled and count in full).
+                        // Both CTAs' bytes complete on the even CTA's barrier, which it arms.
                         if (rank == 0)
                             mbar_arrive_expect_tx(&full[s], 2 * kStageBytes);
                         const uint32_t bar0 = tc::map_to_rank(&full[s], 0);
-#pragma unroll
-                        for (int q = 0; q < KB; ++q) {
-                            tc::tma_load_2d_pair(sA + (s * KB + q) * kABytes, &map_h,
-                                                 (kb + q) * BK, m * BM, bar0);
-                            tc::tma_load_2d_pair(sB + (s * KB + q) * kBBytes, &map_w,
-                                                 (kb + q) * BK, n * BN + rank * (BN / 2), bar0);
-                        }
+                        tc::tma_load_2d_pair(sA + s * kABytes, &map_h, kb * BK, m * BM, bar0);
+                        tc::tma_load_2d_pair(sB + s * kBBytes, &map_w, kb * BK,
+                                             n * BN + rank * (BN / 2), bar0);
                     } else {
                         mbar_arrive_expect_tx(&full[s], kStageBytes);
-#pragma unroll
-                        for (int q = 0; q < KB; ++q) {
-                            tc::tma_load_2d(sA + (s * KB + q) * kABytes, &map_h, (kb + q) * BK,
-                                            m * BM, &full[s]);
-                            tc::tma_load_2d_hint(sB + (s * KB + q) * kBBytes, &map_w,
-                                                 (kb + q) * BK, n * BN, &full[s], pol);
-                        }
-                    }
-                    used[s] = true;
-                    last_ph[s] = ph;
-                    if (++s == kStages) {
-                        s = 0;
-                        ph ^= 1u;
+                        tc::tma_load_2d(sA + s * kABytes, &map_h, kb * BK, m * BM, &full[s]);
+                        tc::tma_load_2d_hint(sB + s * kBBytes, &map_w, kb * BK, n * BN, &full[s],
+                                             pol);
                     }
                 }
+                filled = min(filled + 1, (uint32_t)kStages);
+                if (++s == kStages) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
-            // No copy of this CTA may still be in flight when it exits (in a pair, the even
-            // CTA's barriers count both CTAs' copies, and the odd CTA leaves only after it,
-            // at the final cluster barrier).
-            if (!PAIR || rank == 0)
-                for (int i = 0; i < kStages; ++i)
-                    if (used[i])
-                        mbar_wait(&full[i], last_ph[i], a.status, kDrainLimitNs);
         }
+        // No copy of this CTA may still be in flight when it exits (in a pair, the even
+        // CTA's barriers count both CTAs' copies, and the odd CTA leaves only after it,
+        // at the final cluster barrier).
+        if ((!PAIR || rank == 0) && elect_one())
+            drain_ring(full, kStages, s, ph, filled, a.status);
+        __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0 && (!PAIR || rank == 0)) {
+        if (!PAIR || rank == 0) {
             constexpr uint32_t idesc = tc::idesc_bf16_f32(PAIR ? 2 * BM : BM, BN);
             int s = 0;
             uint32_t ph = 0;
@@ -303,42 +290,40 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int64_t t = first; ok && t < total; t += stride, ++i) {
                 const int acc = i & 1;
                 const uint32_t aph = (uint32_t)(i >> 1) & 1u;
-                if (!wait_or_abort(&tempty[acc], aph ^ 1u, a.status, abort_flag))
+                if (!warp_wait(&tempty[acc], aph ^ 1u, a.status, abort_flag))
                     break;
                 tc::fence_after_sync();
                 const uint32_t d = tmem_base + (uint32_t)acc * kAccStride;
-                for (int kb = 0; kb < a.k_blocks; kb += KB) {
-                    if (!wait_or_abort(&full[s], ph, a.status, abort_flag)) {
+                for (int kb = 0; kb < a.k_blocks; ++kb) {
+                    if (!warp_wait(&full[s], ph, a.status, abort_flag)) {
                         ok = false;
                         break;
                     }
                     tc::fence_after_sync();
-#pragma unroll
-                    for (int q = 0; q < KB; ++q) {
-                        const uint64_t ad = tc::sw128_kmajor_desc(sA + (s * KB + q) * kABytes);
-                        const uint64_t bd = tc::sw128_kmajor_desc(sB + (s * KB + q) * kBBytes);
+                    if (elect_one()) {
+                        const uint64_t ad = tc::sw128_kmajor_desc(sA + s * kABytes);
+                        const uint64_t bd = tc::sw128_kmajor_desc(sB + s * kBBytes);
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k) {  // K = 16 per MMA: +32 B in the row
                             if constexpr (PAIR)
                                 tc::mma_bf16_pair(d, ad + 2u * k, bd + 2u * k, idesc,
-                                                  (kb | q | k) != 0);
+                                                  (kb | k) != 0);
                             else
-                                tc::mma_bf16(d, ad + 2u * k, bd + 2u * k, idesc,
-                                             (kb | q | k) != 0);
+                                tc::mma_bf16(d, ad + 2u * k, bd + 2u * k, idesc, (kb | k) != 0);
                         }
+                        // The stage is free once these MMAs have read it (in a pair, in both
+                        // CTAs: each refills its own half of the pair's operands).
+                        if constexpr (PAIR)
+                            tc::commit_pair_multicast(&empty[s]);
+                        else
+                            tc::commit(&empty[s]);
                     }
-                    // The stage is free once these MMAs have read it (in a pair, in both
-                    // CTAs: each refills its own half of the pair's operands).
-                    if constexpr (PAIR)
-                        tc::commit_pair_multicast(&empty[s]);
-                    else
-                        tc::commit(&empty[s]);
                     if (++s == kStages) {
                         s = 0;
                         ph ^= 1u;
                     }
                 }
-                if (ok) {
+                if (ok && elect_one()) {
                     if constexpr (PAIR)
                         tc::commit_pair_multicast(&tfull[acc]);  // both CTAs' accumulators
                     else
@@ -346,11 +331,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
             // Tensor memory is freed below only after every MMA issued here has completed.
-            if constexpr (PAIR)
-                tc::commit_pair_multicast(done);  // the odd CTA's copy is never waited on
-            else
-                tc::commit(done);
-            mbar_wait(done, 0, a.status, kDrainLimitNs);
+            __syncwarp();
+            if (elect_one()) {
+                if constexpr (PAIR)
+                    tc::commit_pair_multicast(done);  // the odd CTA's copy is never waited on
+                else
+                    tc::commit(done);
+                mbar_wait(done, 0, a.status, kDrainLimitNs);
+            }
         }
         __syncwarp();
     } else {
@@ -561,32 +549,28 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     pdl_wait();  // the packed rows and their count are complete
 
-    const int R = *a.row_count;  // <= kSlabRows: the host takes this variant only then
+    const int R = __shfl_sync(0xFFFFFFFFu, *a.row_count, 0);  // <= kSlabRows: the host takes this variant only then
     const int64_t NT = a.slab_tiles, P = gridDim.x, c = blockIdx.x;
     const int h = a.slab_h;
     const int n_t = R > 0 && c < NT ? (int)((NT - c + P - 1) / P) : 0;  // tiles of this CTA
 
-    if (warp == 0) {
-        if (lane == 0) {
-            const uint64_t pol = make_evict_first_policy();  // W is read once
-            int s = 0;
-            uint32_t ph = 0;
-            uint32_t last_ph[kSlabStages];
-            bool used[kSlabStages];
-            for (int i = 0; i < kSlabStages; ++i)
-                used[i] = false;
-            bool ok = true;
-            // a box's bytes count in full, the part beyond V zero-filled
-            // (K-blocks past H, in the last stage when k_blocks is odd, are zero-filled and
-            // count in full too)
-            const uint32_t bytes = kSlabKB * ((uint32_t)(h * BK * 2) + kSlabBBytes);
-            for (int t = 0; ok && t < n_t; ++t) {
-                const int64_t T = c + (int64_t)t * P;
-                for (int kb = 0; kb < a.k_blocks; kb += kSlabKB) {
-                    if (!wait_or_abort(&empty[s], ph ^ 1u, a.status, abort_flag)) {
-                        ok = false;
-                        break;
-                    }
+    if (warp == 0) {  // warps 0 and 1 whole, one elected lane issuing, as in the tile GEMM
+        const uint64_t pol = make_evict_first_policy();  // W is read once
+        int s = 0;
+        uint32_t ph = 0, filled = 0;
+        bool ok = true;
+        // a box's bytes count in full, the part beyond V zero-filled
+        // (K-blocks past H, in the last stage when k_blocks is odd, are zero-filled and
+        // count in full too)
+        const uint32_t bytes = kSlabKB * ((uint32_t)(h * BK * 2) + kSlabBBytes);
+        for (int t = 0; ok && t < n_t; ++t) {
+            const int64_t T = c + (int64_t)t * P;
+            for (int kb = 0; kb < a.k_blocks; kb += kSlabKB) {
+                if (!warp_wait(&empty[s], ph ^ 1u, a.status, abort_flag)) {
+                    ok = false;
+                    break;
+                }
+                if (elect_one()) {
                     mbar_arrive_expect_tx(&full[s], bytes);
 #pragma unroll
                     for (int q = 0; q < kSlabKB; ++q)
@@ -596,39 +580,38 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int q = 0; q < kSlabKB; ++q)
                         tc::tma_load_2d(sB + (s * kSlabKB + q) * kSlabBBytes, &map_h, (kb + q) * BK,
                                         0, &full[s]);
-                    used[s] = true;
-                    last_ph[s] = ph;
-                    if (++s == kSlabStages) {
-                        s = 0;
-                        ph ^= 1u;
-                    }
+                }
+                filled = min(filled + 1, (uint32_t)kSlabStages);
+                if (++s == kSlabStages) {
+                    s = 0;
+                    ph ^= 1u;
                 }
             }
-            for (int i = 0; i < kSlabStages; ++i)  // none of this CTA's copies in flight at exit
-                if (used[i])
-                    mbar_wait(&full[i], last_ph[i], a.status, kDrainLimitNs);
         }
+        if (elect_one())  // none of this CTA's copies in flight at exit
+            drain_ring(full, kSlabStages, s, ph, filled, a.status);
+        __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_bf16_f32(BM, kSlabRows);
-            int s = 0;
-            uint32_t ph = 0;
-            bool ok = true;
-            for (int t = 0; ok && t < n_t; ++t) {
-                const int acc = t % kSlabAccs;
-                const uint32_t aph = (uint32_t)(t / kSlabAccs) & 1u;
-                if (!wait_or_abort(&tempty[acc], aph ^ 1u, a.status, abort_flag))
+        constexpr uint32_t idesc = tc::idesc_bf16_f32(BM, kSlabRows);
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int t = 0; ok && t < n_t; ++t) {
+            const int acc = t % kSlabAccs;
+            const uint32_t aph = (uint32_t)(t / kSlabAccs) & 1u;
+            if (!warp_wait(&tempty[acc], aph ^ 1u, a.status, abort_flag))
+                break;
+            tc::fence_after_sync();
+            const uint32_t d = tmem_base + (uint32_t)(acc * kSlabRows);
+            for (int kb = 0; kb < a.k_blocks; kb += kSlabKB) {
+                if (!warp_wait(&full[s], ph, a.status, abort_flag)) {
+                    ok = false;
                     break;
+                }
                 tc::fence_after_sync();
-                const uint32_t d = tmem_base + (uint32_t)(acc * kSlabRows);
-                for (int kb = 0; kb < a.k_blocks; kb += kSlabKB) {
-                    if (!wait_or_abort(&full[s], ph, a.status, abort_flag)) {
-                        ok = false;
-                        break;
-                    }
-                    tc::fence_after_sync();
-                    // Rows h..127 of the A stage are stale: those TMEM lanes hold
-                    // meaningless sums that the epilogue skips.
+                // Rows h..127 of the A stage are stale: those TMEM lanes hold
+                // meaningless sums that the epilogue skips.
+                if (elect_one()) {
 #pragma unroll
                     for (int q = 0; q < kSlabKB; ++q) {
                         const uint64_t ad =
@@ -640,14 +623,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                             tc::mma_bf16(d, ad + 2u * k, bd + 2u * k, idesc, (kb | q | k) != 0);
                     }
                     tc::commit(&empty[s]);
-                    if (++s == kSlabStages) {
-                        s = 0;
-                        ph ^= 1u;
-                    }
                 }
-                if (ok)
-                    tc::commit(&tfull[acc]);
+                if (++s == kSlabStages) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
+            if (ok && elect_one())
+                tc::commit(&tfull[acc]);
+        }
+        __syncwarp();
+        if (elect_one()) {
             tc::commit(done);
             mbar_wait(done, 0, a.status, kDrainLimitNs);
         }
