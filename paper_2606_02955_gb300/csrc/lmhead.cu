@@ -766,10 +766,9 @@ constexpr int kWideThreads = 64 + kWideWarps * 32;
 constexpr int kWideChunk = 8;                   // columns an epilogue warp turns at a time
 constexpr size_t kWideBarBytes = 512;
 constexpr int kWidePitch = kWideChunk + 1;      // both ways free of bank conflicts
-constexpr size_t kWideStaging = (size_t)kWideWarps * 32 * kWidePitch * 4;
 constexpr size_t kWideQuarters = (size_t)4 * kWideMaxGroup * (4 + 4 + 1);
 constexpr size_t kWideSmemBytes = 227 * 1024;
-constexpr size_t kWideFixed = kWideBarBytes + kWideStaging + kWideQuarters;
+constexpr size_t kWideFixed = kWideBarBytes + kWideQuarters;
 static_assert((2 * kWideMaxStages + 2 * 4 + 1) * 8 + 8 <= (int)kWideBarBytes, "barriers");
 
 // Tensor maps of the packed rows, box heights 16, 32, ..., 128: entry h / 16 - 1 loads half a
@@ -801,35 +800,107 @@ __device__ __forceinline__ WideCut wide_cut(int R)
 // fills at most half of them and a block has two groups, each leftover item goes to two pairs,
 // one group each.
 struct WideItems {
-    int64_t whole, total;  // items of whole rounds, all items
-    int pairs, pair;
+    // items of whole rounds, all items (B * L * V / 208 < 2^31 keeps them small), this pair
+    int whole, total, pairs, pair;
     bool split;
 
-    __device__ __forceinline__ WideItems(const WideCut &c, int64_t n_w_tiles, int pairs_, int pair_)
+    __device__ __forceinline__ WideItems(const WideCut &c, int n_w_tiles, int pairs_, int pair_)
         : total(n_w_tiles * c.n_blocks), pairs(pairs_), pair(pair_)
     {
-        const int64_t left = total % pairs;
+        const int left = total % pairs;
         whole = total - left;
         split = c.groups == 2 && 2 * left <= pairs;
     }
     // The pair's i-th item: its index, or -1 past the last, and its groups [j0, j1).
-    __device__ __forceinline__ int64_t item(int64_t i, int groups, int &j0, int &j1) const
+    __device__ __forceinline__ int item(int i, int groups, int &j0, int &j1) const
     {
         j0 = 0;
         j1 = groups;
-        const int64_t t = i * pairs + pair;
+        const int t = i * pairs + pair;
         if (t < whole)
             return t;
         if (i != whole / pairs)
             return -1;
         if (!split)
             return t < total ? t : -1;
-        const int64_t u = whole + pair / 2;
+        const int u = whole + pair / 2;
         j0 = pair & 1;
         j1 = j0 + 1;
         return u < total ? u : -1;
     }
 };
+
+// Folds the states (M, S relative to M, first index) of one column from two sets of entries.  Either
+// order gives the same bits.  -inf logits have S = 0; a NaN one leaves S NaN.
+__device__ __forceinline__ void wide_fold(float &M, float &S, uint32_t &I, float M2, float S2,
+                                          uint32_t I2)
+{
+    const bool up = M2 > M;
+    const float hi = up ? M2 : M, lo = up ? M : M2;
+    const float e = lo == -INFINITY ? 0.0f : ex2_mufu((lo - hi) * kLog2e);
+    I = up ? I2 : (M2 == M ? min(I, I2) : I);
+    S = fmaf(up ? S : S2, e, up ? S2 : S);
+    M = hi;
+}
+
+// The column of a 32-column block whose state wide_reduce_block leaves in this lane.
+__device__ __forceinline__ int wide_column(int lane)
+{
+    return (lane >> 3) * 8 + (lane & 3) * 2 + ((lane >> 2) & 1);
+}
+
+// 32 entries (TMEM lanes) x 32 columns in tmem_ld_16x32_async's layout -> per column its maximum
+// M, the sum S of exp(x - M) and the entry 0..31 of the first maximum (255 without a finite
+// logit).  A thread has 4 entries, 8 apart, of each of 8 columns: their state first, then a
+// butterfly over the 8 threads that share them, each step folding one half of the columns and
+// giving the other away: 21 shuffles and no shared memory (turning 8-column blocks in shared
+// memory took 44.2 against 41.4 us at 96 rows, H = 1128, V = 74676).  Entries at or past
+// `entries` lie beyond the vocabulary.
+__device__ __forceinline__ void wide_reduce_block(const float (&x)[2][16], int entries, int lane,
+                                                  float &M, float &S, uint32_t &I)
+{
+    float m[8], s[8];
+    uint32_t id[8];
+    const int e0 = lane >> 2;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        float v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            v[k] = x[k >> 1][(c >> 1) * 4 + (k & 1) * 2 + (c & 1)];
+        if (entries < 32)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                v[k] = e0 + 8 * k < entries ? v[k] : -INFINITY;
+        m[c] = fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]));
+        // exp(x - m) as (x - m) * log2e, exact at any magnitude
+        const float b = m[c] == -INFINITY ? 0.0f : m[c];
+        s[c] = (ex2_mufu((v[0] - b) * kLog2e) + ex2_mufu((v[1] - b) * kLog2e)) +
+               (ex2_mufu((v[2] - b) * kLog2e) + ex2_mufu((v[3] - b) * kLog2e));
+        const int k = v[0] == m[c] ? 0 : v[1] == m[c] ? 8 : v[2] == m[c] ? 16 : 24;
+        id[c] = m[c] == -INFINITY ? 255u : (uint32_t)(e0 + k);
+    }
+#pragma unroll
+    for (int o = 16; o >= 4; o >>= 1) {
+        const bool hi = (lane & o) != 0;
+        const int half = o / 4;
+#pragma unroll
+        for (int c = 0; c < half; ++c) {
+            const float gm = hi ? m[c] : m[c + half], gs = hi ? s[c] : s[c + half];
+            const uint32_t gi = hi ? id[c] : id[c + half];
+            m[c] = hi ? m[c + half] : m[c];
+            s[c] = hi ? s[c + half] : s[c];
+            id[c] = hi ? id[c + half] : id[c];
+            const float rm = __shfl_xor_sync(0xFFFFFFFFu, gm, o);
+            const float rs = __shfl_xor_sync(0xFFFFFFFFu, gs, o);
+            const uint32_t ri = __shfl_xor_sync(0xFFFFFFFFu, gi, o);
+            wide_fold(m[c], s[c], id[c], rm, rs, ri);
+        }
+    }
+    M = m[0];
+    S = s[0];
+    I = id[0];
+}
 
 // bar.red over the epilogue warps: true when every thread's `ok` is true.
 __device__ __forceinline__ bool epilogue_all(bool ok)
@@ -861,8 +932,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     uint64_t *done = tempty + 4;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    float *staging = reinterpret_cast<float *>(fixed + kWideBarBytes);
-    float *q_M = reinterpret_cast<float *>(fixed + kWideBarBytes + kWideStaging);  // [4][256]
+    float *q_M = reinterpret_cast<float *>(fixed + kWideBarBytes);  // [4][256]
     float *q_S = q_M + 4 * kWideMaxGroup;
     uint8_t *q_I = reinterpret_cast<uint8_t *>(q_S + 4 * kWideMaxGroup);
 
@@ -909,12 +979,12 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         uint32_t ph = 0, filled = 0;
         bool ok = true;
         int j0, j1;
-        for (int64_t i = 0; ok; ++i) {
-            const int64_t t = items.item(i, cut.groups, j0, j1);
+        for (int i = 0; ok; ++i) {
+            const int t = items.item(i, cut.groups, j0, j1);
             if (t < 0)
                 break;
-            const int n = (int)(t / cut.n_blocks);
-            const int row0 = (int)(t % cut.n_blocks) * block_rows + rank * (cut.g / 2);
+            const int n = t / cut.n_blocks;
+            const int row0 = t % cut.n_blocks * block_rows + rank * (cut.g / 2);
             const int w_row = n * kWideTile + rank * BM;
             const uint32_t bytes = kABytes + (uint32_t)(j1 - j0) * half_bytes;
             for (int kb = 0; kb < a.k_blocks; ++kb) {
@@ -954,8 +1024,8 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             uint32_t used = 0;  // groups accumulated so far
             bool ok = true;
             int j0, j1;
-            for (int64_t i = 0; ok; ++i) {
-                const int64_t t = items.item(i, cut.groups, j0, j1);
+            for (int i = 0; ok; ++i) {
+                const int t = items.item(i, cut.groups, j0, j1);
                 if (t < 0)
                     break;
                 const bool two = j1 - j0 == 2;
@@ -1040,26 +1110,20 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         }
         __syncwarp();
     } else {
-        // Epilogue: warp w reads TMEM lanes [32 (w % 4), +32) and every third chunk of 8
-        // columns, all of a group's into registers first, which hands the accumulator back after
-        // a few hundred cycles.  A lane's columns are rows of one vocabulary entry, so each 32 x 8
-        // block turns in shared memory: lane l then holds entries 8 (l / 8) + 0..7 of column
-        // l % 8.
-        const int quarter = warp & 3, parity = (warp - 2) >> 2;
+        // Epilogue: warp w reads TMEM lanes [32 (w % 4), +32) and every kWideSplit-th block of 32
+        // columns.
+        const int quarter = warp & 3, third = (warp - 2) >> 2;
         const int et = threadIdx.x - 64;
-        float *block = staging + (warp - 2) * 32 * kWidePitch;
-        const int col = lane & 7, e0 = lane & ~7;
         uint32_t used = 0;
         int j0, j1;
         bool ok = true;
-        for (int64_t i = 0; ok; ++i) {
-            const int64_t t = items.item(i, cut.groups, j0, j1);
+        for (int i = 0; ok; ++i) {
+            const int t = items.item(i, cut.groups, j0, j1);
             if (t < 0)
                 break;
-            const int n = (int)(t / cut.n_blocks);
-            const int blk0 = (int)(t % cut.n_blocks) * block_rows;
+            const int n = t / cut.n_blocks;
+            const int blk0 = t % cut.n_blocks * block_rows;
             const int ent0 = n * kWideTile + rank * BM;
-            const int ent = ent0 + quarter * 32 + lane;
             for (int j = j0; j < j1; ++j, ++used) {
                 const uint32_t buf = used % cut.buffers, turn = used / cut.buffers;
                 const bool got = wait_or_abort(&tfull[buf], turn & 1u, a.status, abort_flag);
@@ -1074,84 +1138,45 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                     tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * cut.g;
                 const int row0 = blk0 + j * cut.g;
                 const int live = min(cut.g, R - row0);  // columns that are rows
-                // Eight chunks (192 of the group's columns) per pass fit the registers.
-                constexpr int kChunks = 8, kPassCols = kChunks * kWideSplit * kWideChunk;
 #pragma unroll 1
-                for (int p0 = 0; p0 < cut.g; p0 += kPassCols) {
-                    float x[kChunks][kWideChunk];
-#pragma unroll
-                    for (int q = 0; q < kChunks; ++q)
-                        if (p0 + (kWideSplit * q + parity) * kWideChunk < live)
-                            tc::tmem_ld_8cols_async(
-                                taddr + p0 + (kWideSplit * q + parity) * kWideChunk, x[q]);
+                for (int c = third * 32; c < live; c += kWideSplit * 32) {
+                    float x[2][16];
+                    if (EPI == kStore) {  // a lane holds 32 rows' logits of its entry
+                        tc::tmem_ld_16cols_async(taddr + c, x[0]);
+                        tc::tmem_ld_16cols_async(taddr + c + 16, x[1]);
+                    } else {
+                        tc::tmem_ld_16x32_async(taddr + c, x[0]);
+                        tc::tmem_ld_16x32_async(taddr + (16u << 16) + c, x[1]);
+                    }
                     tc::tmem_wait_ld();
+                    tc::tie_regs(x[0]);
+                    tc::tie_regs(x[1]);
+                    if (EPI == kStore) {
+                        const int ent = ent0 + quarter * 32 + lane;
+                        const int mine = c + lane < live ? a.row_ids[row0 + c + lane] : 0;
 #pragma unroll
-                    for (int q = 0; q < kChunks; ++q)
-                        tc::tie_regs(x[q]);
-                    if (p0 + kPassCols >= cut.g) {  // the accumulator has been read
-                        tc::fence_before_sync();
-                        __syncwarp();
-                        if (lane == 0) {
-                            if (rank != 0)
-                                tc::mbar_arrive_remote(tc::map_to_rank(&tempty[buf], 0));
-                            else
-                                mbar_arrive(&tempty[buf]);
+                        for (int k = 0; k < 32; ++k) {
+                            const int64_t row = __shfl_sync(0xFFFFFFFFu, mine, k);
+                            if (c + k < live && ent < a.V)
+                                a.logits[row * a.V + ent] = x[k / 16][k % 16];
                         }
+                    } else {
+                        float M, S;
+                        uint32_t I;
+                        wide_reduce_block(x, a.V - (ent0 + quarter * 32), lane, M, S, I);
+                        const int at = quarter * kWideMaxGroup + c + wide_column(lane);
+                        q_M[at] = M;
+                        q_S[at] = S;
+                        q_I[at] = (uint8_t)I;
                     }
-#pragma unroll
-                    for (int q = 0; q < kChunks; ++q) {
-                        const int c = p0 + (kWideSplit * q + parity) * kWideChunk;
-                        if (c >= live)
-                            break;
-                        float(&v)[kWideChunk] = x[q];
-                        if (EPI == kStore) {
-                            const int mine = c + col < live ? a.row_ids[row0 + c + col] : 0;
-#pragma unroll
-                            for (int k = 0; k < kWideChunk; ++k) {
-                                const int64_t row = __shfl_sync(0xFFFFFFFFu, mine, k);
-                                if (c + k < live && ent < a.V)
-                                    a.logits[row * a.V + ent] = v[k];
-                            }
-                            continue;
-                        }
-                        if (ent >= a.V)  // past the vocabulary (the last tile's zero-filled W rows)
-#pragma unroll
-                            for (int k = 0; k < kWideChunk; ++k)
-                                v[k] = -INFINITY;
-                        __syncwarp();  // the block's previous columns have been read
-#pragma unroll
-                        for (int k = 0; k < kWideChunk; ++k)
-                            block[lane * kWidePitch + k] = v[k];
-                        __syncwarp();
-                        float M = -INFINITY;
-#pragma unroll
-                        for (int k = 0; k < kWideChunk; ++k) {
-                            v[k] = block[(e0 + k) * kWidePitch + col];
-                            M = fmaxf(M, v[k]);
-                        }
-                        M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, 8));
-                        M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, 16));
-                        // exp(x - M) as (x - M) * log2e, exact at any magnitude; NaN poisons S, -inf
-                        // adds nothing
-                        const float base = M == -INFINITY ? 0.0f : M;
-                        float S2[2] = {0.0f, 0.0f};
-                        int first = 255;
-#pragma unroll
-                        for (int k = kWideChunk - 1; k >= 0; --k) {
-                            first = v[k] == M ? e0 + k : first;
-                            S2[k & 1] += ex2_mufu((v[k] - base) * kLog2e);
-                        }
-                        float S = S2[0] + S2[1];
-                        S += __shfl_xor_sync(0xFFFFFFFFu, S, 8);
-                        S += __shfl_xor_sync(0xFFFFFFFFu, S, 16);
-                        first = min(first, __shfl_xor_sync(0xFFFFFFFFu, first, 8));
-                        first = min(first, __shfl_xor_sync(0xFFFFFFFFu, first, 16));
-                        if (e0 == 0) {
-                            q_M[quarter * kWideMaxGroup + c + col] = M;
-                            q_S[quarter * kWideMaxGroup + c + col] = S;
-                            q_I[quarter * kWideMaxGroup + c + col] = (uint8_t)first;
-                        }
-                    }
+                }
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) {
+                    if (rank != 0)
+                        tc::mbar_arrive_remote(tc::map_to_rank(&tempty[buf], 0));
+                    else
+                        mbar_arrive(&tempty[buf]);
                 }
                 if (EPI == kReduce) {
                     asm volatile("barrier.cta.sync 2, %0;" ::"n"(kWideWarps * 32) : "memory");

@@ -249,15 +249,32 @@ __device__ __forceinline__ void tmem_ld_32cols(uint32_t taddr, float (&v)[32])
         v[i] = __uint_as_float(r[i]);
 }
 
-// 8 columns as tmem_ld_32cols, without the wait: the values are there once tmem_wait_ld() has
+// 16 columns as tmem_ld_32cols, without the wait: the values are there once tmem_wait_ld() has
 // run and tie_regs() has been called on them after it.
-__device__ __forceinline__ void tmem_ld_8cols_async(uint32_t taddr, float (&v)[8])
+__device__ __forceinline__ void tmem_ld_16cols_async(uint32_t taddr, float (&v)[16])
 {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]),
-                   "=f"(v[6]), "=f"(v[7])
-                 : "r"(taddr)
-                 : "memory");
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
+          "=f"(v[7]), "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]),
+          "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+        : "r"(taddr)
+        : "memory");
+}
+
+// 32 columns of 16 TMEM lanes, without the wait (as above): v[4 b + 2 j + c] of thread t is lane
+// t / 4 + 8 j, column 8 b + 2 (t % 4) + c.
+__device__ __forceinline__ void tmem_ld_16x32_async(uint32_t taddr, float (&v)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
+          "=f"(v[7]), "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]),
+          "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+        : "r"(taddr)
+        : "memory");
 }
 
 __device__ __forceinline__ void tmem_wait_ld()
@@ -265,13 +282,16 @@ __device__ __forceinline__ void tmem_wait_ld()
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ void tie_regs(float (&v)[8])
+template <int N>
+__device__ __forceinline__ void tie_regs(float (&v)[N])
 {
-    asm volatile(""
-                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]),
-                   "+f"(v[6]), "+f"(v[7])
-                 :
-                 : "memory");
+#pragma unroll
+    for (int i = 0; i < N; i += 8)
+        asm volatile(""
+                     : "+f"(v[i]), "+f"(v[i + 1]), "+f"(v[i + 2]), "+f"(v[i + 3]), "+f"(v[i + 4]),
+                       "+f"(v[i + 5]), "+f"(v[i + 6]), "+f"(v[i + 7])
+                     :
+                     : "memory");
 }
 
 }  // namespace tc
