@@ -247,53 +247,81 @@ __device__ __forceinline__ float rebase(float S, float a, float b)
     return S != 0.0f ? S * ex2_mufu((a - b) * kLog2e) : 0.0f;
 }
 
-// Position result from its units, folded in unit order (a fixed order, so identical rows
-// give identical bits): c = min(1/S, 1) (the max term alone is 1) and x_hat = the first
-// index attaining the max; c = NaN, x_hat = -1 when the row holds a NaN or its maximum is
-// +inf or -inf.
+// Results of P positions from their units, folded in unit order, eight at a time (a fixed order,
+// so identical rows give identical bits): c = min(1/S, 1) (the max term alone is 1) and x_hat =
+// the first index attaining the max; c = NaN, x_hat = -1 when the row holds a NaN or its maximum
+// is +inf or -inf.  p[i] is null for a position without partials (c and tok untouched).  The P
+// positions' loads are in flight together.
+template <int P>
+__device__ __forceinline__ void combine_positions(const UnitPartial *const (&p)[P], int upr,
+                                                  float (&c)[P], int32_t (&tok)[P])
+{
+    constexpr int U = 8;
+    float M[P], S[P];
+    uint32_t idx[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+        M[i] = -__int_as_float(0x7F800000);
+        S[i] = 0.0f;
+        idx[i] = kNoIdx;
+    }
+    for (int j0 = 0; j0 < upr; j0 += U) {
+        const int cnt = upr - j0 < U ? upr - j0 : U;
+        float Mj[P][U], Sj[P][U];
+        uint32_t Ij[P][U];
+#pragma unroll
+        for (int i = 0; i < P; ++i)
+#pragma unroll
+            for (int j = 0; j < U; ++j)
+                if (j < cnt && p[i] != nullptr) {
+                    const int4 r = __ldcg(reinterpret_cast<const int4 *>(p[i] + j0 + j));
+                    Mj[i][j] = __int_as_float(r.x);
+                    Sj[i][j] = __int_as_float(r.y);
+                    Ij[i][j] = (uint32_t)r.z;
+                }
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+            if (p[i] == nullptr)
+                continue;
+            float Mb = M[i];
+#pragma unroll
+            for (int j = 0; j < U; ++j)
+                if (j < cnt)
+                    Mb = fmaxf(Mb, Mj[i][j]);
+            float Sb = rebase(S[i], M[i], Mb);
+            uint32_t ib = (M[i] == Mb) ? idx[i] : kNoIdx;
+#pragma unroll
+            for (int j = 0; j < U; ++j)
+                if (j < cnt) {
+                    Sb += rebase(Sj[i][j], Mj[i][j], Mb);
+                    if (Mj[i][j] == Mb && ib == kNoIdx)
+                        ib = Ij[i][j];
+                }
+            M[i] = Mb;
+            S[i] = Sb;
+            idx[i] = ib;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+        if (p[i] == nullptr)
+            continue;
+        const bool finite = fabsf(M[i]) <= 3.402823466e38f && fabsf(S[i]) <= 3.402823466e38f;
+        const bool ok = finite && S[i] > 0.0f && idx[i] != kNoIdx;
+        tok[i] = ok ? (int32_t)idx[i] : -1;
+        c[i] = ok ? fminf(1.0f / S[i], 1.0f) : __int_as_float(0x7FC00000);
+    }
+}
+
 __device__ __forceinline__ void combine_position(const UnitPartial *p, int upr, float &c,
                                                  int32_t &tok)
 {
-    float Mj[8], Sj[8];
-    uint32_t Ij[8];
-    float M = -__int_as_float(0x7F800000);
-    float S = 0.0f;
-    uint32_t idx = kNoIdx;
-    for (int j0 = 0; j0 < upr; j0 += 8) {
-        const int cnt = upr - j0 < 8 ? upr - j0 : 8;
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            if (j < cnt) {
-                const int4 r = __ldcg(reinterpret_cast<const int4 *>(p + j0 + j));
-                Mj[j] = __int_as_float(r.x);
-                Sj[j] = __int_as_float(r.y);
-                Ij[j] = (uint32_t)r.z;
-            }
-        float Mb = M;
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            if (j < cnt)
-                Mb = fmaxf(Mb, Mj[j]);
-        float Sb = rebase(S, M, Mb);
-        uint32_t ib = (M == Mb) ? idx : kNoIdx;
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            if (j < cnt) {
-                Sb += rebase(Sj[j], Mj[j], Mb);
-                if (Mj[j] == Mb && ib == kNoIdx)
-                    ib = Ij[j];
-            }
-        M = Mb;
-        S = Sb;
-        idx = ib;
-    }
-    c = __int_as_float(0x7FC00000);
-    tok = -1;
-    const bool finite = fabsf(M) <= 3.402823466e38f && fabsf(S) <= 3.402823466e38f;
-    if (!finite || !(S > 0.0f) || idx == kNoIdx)
-        return;
-    tok = (int32_t)idx;
-    c = fminf(1.0f / S, 1.0f);
+    const UnitPartial *const pp[1] = {p};
+    float cc[1];
+    int32_t tt[1];
+    combine_positions(pp, upr, cc, tt);
+    c = cc[0];
+    tok = tt[0];
 }
 
 // Programmatic dependent launch: the dependent grid's wait for the primary grid's results,

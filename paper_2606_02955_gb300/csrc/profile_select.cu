@@ -1,9 +1,9 @@
 // profile_select.cu -- steps a2-a5 of the selection for one batch row per CTA (paper
 // Algorithm 1: sort, scan, select, reveal):
-//   a2  sort the masked (c, position) pairs by c descending, position ascending: one 64-bit
-//       key per thread; rows of at most 32 positions (one warp) by rank counting (each key's
-//       rank is the number of smaller keys, 32 independent shuffles), longer rows by a
-//       bitonic network (warp shuffles for partner distance < 32, shared memory above);
+//   a2  sort the masked (c, position) pairs by c descending, position ascending, as 64-bit
+//       keys; rows of at most 32 positions (one warp) by rank counting (each key's rank is the
+//       number of smaller keys, 32 independent shuffles), longer rows by a bitonic network of
+//       two keys per thread (shuffles and registers up to distance 32, shared memory above);
 //   a3  prefix sums over the sorted order in 64-bit fixed point (units of 2^-52, exact and
 //       independent of the summation order; warp shuffles, then across warps):
 //       P_n = sum_{j<=n} (1 - c_(j)), so L_n = max{0, 1 - P_n} (= sum c - (n-1), Sec. 3),
@@ -52,63 +52,100 @@ __device__ __forceinline__ float key_conf(uint64_t key)
     return __uint_as_float(kOneBits - (uint32_t)(key >> 32));
 }
 
-template <int T>
-__device__ __forceinline__ uint64_t bitonic_sort(uint64_t key, uint64_t *sk)
+// A row of more than 32 positions is held by W warps of K keys per thread: element
+// (w K + r) 32 + lane is key[r] of that lane of warp w.
+//
+// Bitonic sort of the N = 32 K W keys.  Partners up to 16 apart are shuffled, 32 (and 64, with
+// K = 4) apart are registers of one thread, and only those 32 K or more apart go through shared
+// memory (two halves of buf[2 N] in turn, one barrier per stage).  What bounds the kernels is the
+// latency of this chain and, after the vocab reduction, of the partials' loads, so the selection
+// takes two keys per thread: four put two rounds of loads in a row (12.4 us after the reduction
+// at L = 1024 and 5 units per row, two keys 8.9, one key 9.8 and, with the earlier one-key
+// kernel's two barriers per stage, 11.7), and one key needs 15 shared stages for 1024 positions
+// where two need 10.  On given confidences: 1000 positions 9.6 -> 6.6 us, 256 4.0 -> 3.3, 61 2.7
+// -> 2.3.  The terms kernel loads one value per position: four keys at 1024 (14.8 -> 8.3 us; 9.2
+// with two), two below (256 5.2 -> 3.7).
+template <int W, int K>
+__device__ __forceinline__ void sort_keys(uint64_t (&key)[K], uint64_t *buf)
 {
-    const int t = threadIdx.x;
+    constexpr int N = 32 * K * W;
+    const int lane = threadIdx.x & 31;
+    const int idx0 = (int)(threadIdx.x >> 5) * 32 * K + lane;
+    int turn = 0;  // the half of buf[2 N] in use
 #pragma unroll 1
-    for (int k = 2; k <= T; k <<= 1) {
+    for (int k = 2; k <= N; k <<= 1) {
+        bool up[K];  // the element's run of k is sorted upwards
+#pragma unroll
+        for (int r = 0; r < K; ++r)
+            up[r] = ((idx0 + 32 * r) & k) == 0;
+        if constexpr (W > 1) {
 #pragma unroll 1
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            uint64_t other;
-            if (j >= 32) {
-                sk[t] = key;
+            for (int j = k >> 1; j >= 32 * K; j >>= 1) {
+#pragma unroll
+                for (int r = 0; r < K; ++r)
+                    buf[turn + idx0 + 32 * r] = key[r];
                 __syncthreads();
-                other = sk[t ^ j];
-                __syncthreads();
-            } else {
-                other = __shfl_xor_sync(0xFFFFFFFFu, key, j);
+#pragma unroll
+                for (int r = 0; r < K; ++r) {
+                    const uint64_t other = buf[turn + ((idx0 + 32 * r) ^ j)];
+                    if ((other < key[r]) == (((idx0 & j) == 0) == up[r]))
+                        key[r] = other;
+                }
+                turn = N - turn;
             }
-            const bool ascending = (t & k) == 0;
-            const bool lower = (t & j) == 0;
-            const uint64_t lo = key < other ? key : other;
-            const uint64_t hi = key < other ? other : key;
-            key = (lower == ascending) ? lo : hi;
         }
+#pragma unroll
+        for (int jr = K / 2; jr >= 1; jr >>= 1)
+            if (k >= 64 * jr)
+#pragma unroll
+                for (int r = 0; r < K; ++r)
+                    if ((r & jr) == 0 && (key[r + jr] < key[r]) == up[r]) {
+                        const uint64_t t = key[r];
+                        key[r] = key[r + jr];
+                        key[r + jr] = t;
+                    }
+#pragma unroll 1
+        for (int j = k >= 32 ? 16 : k >> 1; j > 0; j >>= 1)
+#pragma unroll
+            for (int r = 0; r < K; ++r) {
+                const uint64_t other = __shfl_xor_sync(0xFFFFFFFFu, key[r], j);
+                if ((other < key[r]) == (((lane & j) == 0) == up[r]))
+                    key[r] = other;
+            }
     }
-    return key;
 }
 
-template <int T, typename V>
-__device__ __forceinline__ V block_inclusive_scan(V v, V *warp_tot)
+// Inclusive prefix sums of v over the elements in order.
+template <int W, int K, typename V>
+__device__ __forceinline__ void scan_elements(V (&v)[K], V *warp_tot)
 {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const V u = __shfl_up_sync(0xFFFFFFFFu, v, o);
-        if (lane >= o)
-            v += u;
-    }
-    if constexpr (T > 32) {
-        if (lane == 31)
-            warp_tot[w] = v;
-        __syncthreads();
-        if (w == 0) {
-            V x = lane < T / 32 ? warp_tot[lane] : V(0);
+    for (int o = 1; o < 32; o <<= 1)
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const V u = __shfl_up_sync(0xFFFFFFFFu, x, o);
-                if (lane >= o)
-                    x += u;
-            }
-            if (lane < T / 32)
-                warp_tot[lane] = x;  // inclusive over warps
+        for (int r = 0; r < K; ++r) {
+            const V u = __shfl_up_sync(0xFFFFFFFFu, v[r], o);
+            if (lane >= o)
+                v[r] += u;
         }
+    V base = V(0);
+    if constexpr (W > 1) {
+        V total = V(0);
+#pragma unroll
+        for (int r = 0; r < K; ++r)
+            total += __shfl_sync(0xFFFFFFFFu, v[r], 31);
+        if (lane == 0)
+            warp_tot[w] = total;
         __syncthreads();
-        if (w > 0)
-            v += warp_tot[w - 1];
+        for (int i = 0; i < w; ++i)
+            base += warp_tot[i];
     }
-    return v;
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        const V last = __shfl_sync(0xFFFFFFFFu, v[r], 31);
+        v[r] += base;
+        base += last;
+    }
 }
 
 // The rule's acceptance of prefix size n, from c_(n) (fp32), v = 1 - c_(n) and the prefix
@@ -127,50 +164,41 @@ __device__ __forceinline__ bool rule_accepts(int mode, int n, float cn, int64_t 
     return cn >= tau_f;  // threshold: c_(n) >= tau
 }
 
-template <int T>
-__device__ __forceinline__ int block_max(int v, int *warp_red)
+template <int W, int K>
+__global__ void __launch_bounds__(32 * W) profile_select_kernel(const ProfileSelectArgs a,
+                                                                 int64_t bound, float tau_f)
 {
-    v = __reduce_max_sync(0xFFFFFFFFu, v);
-    if constexpr (T > 32) {
-        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-        __syncthreads();  // warp_red may still be read from an earlier use
-        if (lane == 0)
-            warp_red[w] = v;
-        __syncthreads();
-        int x = lane < T / 32 ? warp_red[lane] : 0;
-        v = __reduce_max_sync(0xFFFFFFFFu, x);
-    }
-    return v;
-}
+    constexpr int N = 32 * K * W;
+    __shared__ uint64_t sk[W > 1 ? 2 * N : 1];
+    __shared__ int32_t s_tok[N];
+    __shared__ int64_t warp_tot[W];
+    __shared__ int warp_m[W], warp_n[W];
+    constexpr unsigned kFull = 0xFFFFFFFFu;
 
-template <int T>
-__global__ void __launch_bounds__(T) profile_select_kernel(const ProfileSelectArgs a,
-                                                            int64_t bound, float tau_f)
-{
-    __shared__ uint64_t sk[T > 32 ? T : 1];
-    __shared__ int32_t s_tok[T];
-    __shared__ int64_t warp_tot[32];
-    __shared__ int warp_red[32];
-
-    const int t = threadIdx.x;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int pos0 = w * 32 * K + lane;  // this thread's positions: pos0 + 32 r
     const int L = a.L;
     const int64_t base = (int64_t)blockIdx.x * L;
 
-    // (c, x_hat) of this thread's position: folded from the vocab reduction's unit
+    // (c, x_hat) of this thread's positions: folded from the vocab reduction's unit
     // partials, or read from the given arrays.  Launched as a programmatic dependent: the
     // producer of the partials or confidences has completed past the launch wait.  As in the
-    // warp kernel, after the vocab reduction the mask byte and the allowance are loaded
+    // warp kernel, after the vocab reduction the mask bytes and the allowances are loaded
     // before that wait (their writers completed before the reduction passed its own wait,
     // and the reduction writes neither); the partials or confidences and the status word
     // after it, all issued before any is used.
-    const bool in_row = t < L;
     const bool early = a.partials != nullptr;
-    uint8_t mask_byte = 0;
-    float eta = (float)a.eta;
+    uint8_t mask_byte[K];
+    float eta[K];
     auto load_row_inputs = [&]() {
-        mask_byte = in_row ? __ldcg(a.mask + base + t) : (uint8_t)0;
-        if (a.mode == kModeRobust && a.eta_pos != nullptr && in_row)
-            eta = fmaxf(__ldcg(a.eta_pos + base + t), 0.0f);  // negative or NaN: 0
+#pragma unroll
+        for (int r = 0; r < K; ++r) {
+            const int pos = pos0 + 32 * r;
+            mask_byte[r] = pos < L ? __ldcg(a.mask + base + pos) : (uint8_t)0;
+            eta[r] = (float)a.eta;
+            if (a.mode == kModeRobust && a.eta_pos != nullptr && pos < L)
+                eta[r] = fmaxf(__ldcg(a.eta_pos + base + pos), 0.0f);  // negative or NaN: 0
+        }
     };
     if (threadIdx.x == 0)
         pdl_launch_dependents();  // a following vocab reduction may start its prologue
@@ -180,65 +208,109 @@ __global__ void __launch_bounds__(T) profile_select_kernel(const ProfileSelectAr
     if (!early)
         load_row_inputs();
     const bool dev_err = a.status != nullptr && (__ldcg(a.status) & kDevStatTimeout) != 0;
-    const bool masked = mask_byte != 0;
-    float c = 0.0f;
-    int32_t tok = -1;
-    if (in_row) {
-        if (a.partials != nullptr) {
-            combine_position(a.partials + (base + t) * a.units_per_row, a.units_per_row, c,
-                             tok);
-        } else {
-            c = __ldcg(a.conf + base + t);
-            tok = __ldcg(a.tok + base + t);
-        }
+    float c[K];
+    int32_t tok[K];
+    if (a.partials != nullptr) {
+        const int upr = a.units_per_row;
+        const UnitPartial *p[K];
+#pragma unroll
+        for (int r = 0; r < K; ++r)  // unmasked positions have none
+            p[r] = mask_byte[r] != 0 ? a.partials + (base + pos0 + 32 * r) * upr : nullptr;
+        combine_positions(p, upr, c, tok);
+    } else {
+#pragma unroll
+        for (int r = 0; r < K; ++r)
+            if (pos0 + 32 * r < L) {
+                c[r] = __ldcg(a.conf + base + pos0 + 32 * r);
+                tok[r] = __ldcg(a.tok + base + pos0 + 32 * r);
+            }
     }
-    if (!masked) {
-        c = 0.0f;
-        tok = -1;
-    }
-    s_tok[t] = tok;
-    if (a.partials != nullptr && a.next_unit != nullptr && blockIdx.x == 0 && t == 0)
+    if (a.partials != nullptr && a.next_unit != nullptr && blockIdx.x == 0 && threadIdx.x == 0)
         *a.next_unit = 0;  // the vocab reduction before this kernel has finished
-    const bool bad = masked && !(c > 0.0f && c <= 1.0f);  // NaN fails both
-    // The robust rule ranks and scans lower confidences max{0, c - eta} (App. C).
-    float c_rank = c;
-    if (a.mode == kModeRobust && masked && !bad)
-        c_rank = fmaxf(0.0f, c - eta);
-    uint64_t key = t < L ? make_key(masked, c_rank, t) : kPadKey;
+    uint64_t key[K];
+    int m = 0;
+    bool any_bad = false;
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        const int pos = pos0 + 32 * r;
+        const bool masked = mask_byte[r] != 0;
+        if (!masked) {
+            c[r] = 0.0f;
+            tok[r] = -1;
+        }
+        s_tok[pos] = tok[r];
+        const bool bad = masked && !(c[r] > 0.0f && c[r] <= 1.0f);  // NaN fails both
+        // The robust rule ranks and scans lower confidences max{0, c - eta} (App. C).
+        float c_rank = c[r];
+        if (a.mode == kModeRobust && masked && !bad)
+            c_rank = fmaxf(0.0f, c[r] - eta[r]);
+        key[r] = pos < L ? make_key(masked, c_rank, pos) : kPadKey;
+        m += __popc(__ballot_sync(kFull, masked));
+        any_bad |= __any_sync(kFull, bad) != 0;
+    }
+    if constexpr (W > 1) {
+        if (lane == 0)
+            warp_m[w] = any_bad ? -1 : m;
+        __syncthreads();
+        m = 0;
+        any_bad = false;
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            any_bad |= warp_m[i] < 0;
+            m += warp_m[i];  // meaningless, and unused, with a bad position
+        }
+    } else {
+        __syncwarp();
+    }
 
-    const int m = __syncthreads_count(masked);
-    const int any_bad = __syncthreads_or(bad);
+    sort_keys<W, K>(key, sk);
 
-    key = bitonic_sort<T>(key, sk);
-
-    // Thread t now holds the (t+1)-th most confident masked position when t < m.
-    const int n = t + 1;
-    const bool live = t < m;
-    const float cn = live ? key_conf(key) : 1.0f;
-    const int64_t v = live ? one_minus_fixed(cn) : 0;
-    const int64_t P = block_inclusive_scan<T>(v, warp_tot);
-    const bool ok = live && rule_accepts(a.mode, n, cn, v, P, bound, tau_f);
-    int nstar = block_max<T>(ok ? n : 0, warp_red);
+    // This thread now holds, as key[r], the n-th most confident masked position when n <= m.
+    int64_t v[K], P[K];
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        v[r] = pos0 + 32 * r < m ? one_minus_fixed(key_conf(key[r])) : 0;
+        P[r] = v[r];
+    }
+    scan_elements<W, K>(P, warp_tot);
+    int nstar = 0;
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        const int n = pos0 + 32 * r + 1;
+        if (n <= m && rule_accepts(a.mode, n, key_conf(key[r]), v[r], P[r], bound, tau_f))
+            nstar = n;  // n grows with r
+    }
+    nstar = __reduce_max_sync(kFull, nstar);
+    if constexpr (W > 1) {
+        if (lane == 0)
+            warp_n[w] = nstar;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            nstar = max(nstar, warp_n[i]);
+    }
     if (m > 0 && nstar == 0)
         nstar = 1;  // progress convention
     if (any_bad) {
         nstar = -1;
-        if (t == 0 && a.status != nullptr)
+        if (threadIdx.x == 0 && a.status != nullptr)
             atomicOr(a.status, kDevStatNonfinite);
     }
     if (dev_err)
         nstar = -2;
 
-    if (t < L) {
-        const int pos = (int)(key & 0xFFFFFFFFu);
-        const bool commit = t < nstar;  // nstar <= m, so only masked keys qualify
-        a.out_commit[base + pos] = commit ? 1 : 0;
-        if (commit) {
-            a.out_tokens[base + pos] = s_tok[pos];
-            a.mask[base + pos] = 0;
+#pragma unroll
+    for (int r = 0; r < K; ++r)
+        if (pos0 + 32 * r < L) {
+            const int pos = (int)(key[r] & 0xFFFFFFFFu);
+            const bool commit = pos0 + 32 * r < nstar;  // nstar <= m: only masked keys qualify
+            a.out_commit[base + pos] = commit ? 1 : 0;
+            if (commit) {
+                a.out_tokens[base + pos] = s_tok[pos];
+                a.mask[base + pos] = 0;
+            }
         }
-    }
-    if (t == 0)
+    if (threadIdx.x == 0)
         a.out_n[blockIdx.x] = nstar;
 }
 
@@ -356,43 +428,95 @@ __global__ void __launch_bounds__(32) profile_select_warp_kernel(const ProfileSe
 // inclusive scan S_n = sum_{j<=n} c_(j), and at rank n: G_n = max{0, S_n - (n-1)} - (1 - c_(n)),
 // F_n = (n+1) c_(n) - n and B_n = S_n - n c_(n) (= sum_{j<n} (c_(j) - c_(n))); and the
 // effective factor f_eff(n) = 1 - delta + B_n of Remark adaptive-factor.
-template <int T>
-__global__ void __launch_bounds__(T) profile_terms_kernel(const ProfileTermsArgs a)
+template <int W, int K>
+__global__ void __launch_bounds__(32 * W) profile_terms_kernel(const ProfileTermsArgs a)
 {
-    __shared__ uint64_t sk[T > 32 ? T : 1];
-    __shared__ double warp_tot[32];
-    const int t = threadIdx.x;
+    constexpr int N = 32 * K * W;
+    __shared__ uint64_t sk[W > 1 ? 2 * N : 1];
+    __shared__ double warp_tot[W];
+    __shared__ int warp_m[W];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int pos0 = w * 32 * K + lane;
     const int L = a.L;
     const int64_t base = (int64_t)blockIdx.x * L;
-    const bool masked = t < L && a.mask[base + t] != 0;
-    const float c = masked ? a.conf[base + t] : 0.0f;
-    uint64_t key = t < L ? make_key(masked, c, t) : kPadKey;
-    const int m = __syncthreads_count(masked);
-    key = bitonic_sort<T>(key, sk);
-    const bool live = t < m;
-    const double cn = live ? (double)key_conf(key) : 0.0;
-    const double S = block_inclusive_scan<T>(cn, warp_tot);
-    if (t >= L)
-        return;
-    const double n = (double)(t + 1);
+    pdl_wait();  // the confidences and the mask are written
+    if (threadIdx.x == 0)
+        pdl_launch_dependents();
+    uint64_t key[K];
+    int m = 0;
+    uint8_t mask_byte[K];
+    float c[K];
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        const int pos = pos0 + 32 * r;
+        mask_byte[r] = pos < L ? a.mask[base + pos] : (uint8_t)0;
+        c[r] = pos < L ? a.conf[base + pos] : 0.0f;
+    }
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        const int pos = pos0 + 32 * r;
+        const bool masked = mask_byte[r] != 0;
+        key[r] = pos < L ? make_key(masked, masked ? c[r] : 0.0f, pos) : kPadKey;
+        m += __popc(__ballot_sync(0xFFFFFFFFu, masked));
+    }
+    if constexpr (W > 1) {
+        if (lane == 0)
+            warp_m[w] = m;
+        __syncthreads();
+        m = 0;
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            m += warp_m[i];
+    }
+    sort_keys<W, K>(key, sk);
+    double cn[K], S[K];
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        cn[r] = pos0 + 32 * r < m ? (double)key_conf(key[r]) : 0.0;
+        S[r] = cn[r];
+    }
+    scan_elements<W, K>(S, warp_tot);
     const double nan = __longlong_as_double(0x7FF8000000000000ll);
-    if (a.out_G != nullptr)
-        a.out_G[base + t] = live ? fmax(0.0, S - (n - 1.0)) - (1.0 - cn) : nan;
-    if (a.out_F != nullptr)
-        a.out_F[base + t] = live ? (n + 1.0) * cn - n : nan;
-    if (a.out_B != nullptr)
-        a.out_B[base + t] = live ? S - n * cn : nan;
-    if (a.out_feff != nullptr)
-        a.out_feff[base + t] = live ? 1.0 - a.delta + (S - n * cn) : nan;
-    if (a.out_order != nullptr)
-        a.out_order[base + t] = live ? (int32_t)(key & 0xFFFFFFFFu) : -1;
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        const int t = pos0 + 32 * r;
+        if (t >= L)
+            continue;
+        const bool live = t < m;
+        double G = nan, F = nan, Bn = nan, fe = nan;
+        if (live) {  // fp64 runs at two lanes per clock and SM: none for the ranks past m
+            const double n = (double)(t + 1);
+            G = fmax(0.0, S[r] - (n - 1.0)) - (1.0 - cn[r]);
+            F = (n + 1.0) * cn[r] - n;
+            Bn = S[r] - n * cn[r];
+            fe = 1.0 - a.delta + Bn;
+        }
+        if (a.out_G != nullptr)
+            a.out_G[base + t] = G;
+        if (a.out_F != nullptr)
+            a.out_F[base + t] = F;
+        if (a.out_B != nullptr)
+            a.out_B[base + t] = Bn;
+        if (a.out_feff != nullptr)
+            a.out_feff[base + t] = fe;
+        if (a.out_order != nullptr)
+            a.out_order[base + t] = live ? (int32_t)(key[r] & 0xFFFFFFFFu) : -1;
+    }
 }
 
-template <int T>
+template <int W, int K>
 cudaError_t launch_terms_t(const ProfileTermsArgs &a, cudaStream_t stream)
 {
-    profile_terms_kernel<T><<<a.B, T, 0, stream>>>(a);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)a.B);
+    cfg.blockDim = dim3(32 * W);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, profile_terms_kernel<W, K>, a);
 }
 
 template <typename Kernel>
@@ -428,29 +552,29 @@ cudaError_t launch_profile_select(const ProfileSelectArgs &a, cudaStream_t strea
     if (a.L <= 32)
         return launch_select(profile_select_warp_kernel, 32, a, bound, tau_f, stream);
     if (a.L <= 64)
-        return launch_select(profile_select_kernel<64>, 64, a, bound, tau_f, stream);
+        return launch_select(profile_select_kernel<1, 2>, 32, a, bound, tau_f, stream);
     if (a.L <= 128)
-        return launch_select(profile_select_kernel<128>, 128, a, bound, tau_f, stream);
+        return launch_select(profile_select_kernel<2, 2>, 64, a, bound, tau_f, stream);
     if (a.L <= 256)
-        return launch_select(profile_select_kernel<256>, 256, a, bound, tau_f, stream);
+        return launch_select(profile_select_kernel<4, 2>, 128, a, bound, tau_f, stream);
     if (a.L <= 512)
-        return launch_select(profile_select_kernel<512>, 512, a, bound, tau_f, stream);
-    return launch_select(profile_select_kernel<1024>, 1024, a, bound, tau_f, stream);
+        return launch_select(profile_select_kernel<8, 2>, 256, a, bound, tau_f, stream);
+    return launch_select(profile_select_kernel<16, 2>, 512, a, bound, tau_f, stream);
 }
 
 cudaError_t launch_profile_terms(const ProfileTermsArgs &a, cudaStream_t stream)
 {
     if (a.L <= 32)
-        return launch_terms_t<32>(a, stream);
+        return launch_terms_t<1, 1>(a, stream);
     if (a.L <= 64)
-        return launch_terms_t<64>(a, stream);
+        return launch_terms_t<1, 2>(a, stream);
     if (a.L <= 128)
-        return launch_terms_t<128>(a, stream);
+        return launch_terms_t<2, 2>(a, stream);
     if (a.L <= 256)
-        return launch_terms_t<256>(a, stream);
+        return launch_terms_t<4, 2>(a, stream);
     if (a.L <= 512)
-        return launch_terms_t<512>(a, stream);
-    return launch_terms_t<1024>(a, stream);
+        return launch_terms_t<8, 2>(a, stream);
+    return launch_terms_t<8, 4>(a, stream);
 }
 
 }  // namespace fdllm
