@@ -7,9 +7,9 @@
 //
 // Launch sequence on one stream (all rows of one step), chained by programmatic dependent
 // launches:
-//   1. compact_rows_kernel   the masked rows' indices and their count (one CTA)
-//   2. gather_rows_kernel    the masked rows' hidden states, packed [R, H] (TMA-friendly)
-//   3. lmhead_gemm_kernel    persistent tcgen05 GEMM: warp 0 issues TMA loads into a ring of
+//   1. pack_rows_kernel      the masked rows' indices, their count and their hidden states,
+//                            packed [R, H] (TMA-friendly)
+//   2. lmhead_gemm_kernel    persistent tcgen05 GEMM: warp 0 issues TMA loads into a ring of
 //                            stages, warp 1 issues tcgen05.mma into one of two TMEM
 //                            accumulators, warps 2-5 reduce (or store) the other one; solo
 //                            or CTA-pair (cta_group::2) variants
@@ -17,9 +17,9 @@
 //                            each CTA streams one vocabulary slab, one partial per row
 //      lmhead_wide_kernel    (up to 896 rows) the operands swapped on a CTA pair, W as the
 //                            M = 256 side and up to 256 (or 320) rows as N
-//   4. combine_rows_kernel   four warps per row fold its tile (or slab) partials in a fixed
-//      combine_wide_kernel   order; the wide variant's, laid out by tile, four rows per CTA
-//   5. profile_select        steps a2-a5 on the confidences (profile_select.cu)
+//   3. combine_rows_kernel   four warps per row fold its tile (or slab) partials in a fixed
+//                            order
+//   4. profile_select        steps a2-a5 on the confidences (profile_select.cu)
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -87,7 +87,7 @@ struct TileCfg {
 };
 
 struct GemmArgs {
-    const int32_t *row_count;  // R, written by compact_rows_kernel
+    const int32_t *row_count;  // R, written by pack_rows_kernel
     const int32_t *row_ids;    // [R] global row (b * L + l) of each packed row
     int32_t V;
     int32_t n_tiles;           // partials per row: ceil(V / BN), or the slab variant's grid
@@ -95,8 +95,7 @@ struct GemmArgs {
     int32_t slab_tiles;        // slab variant: vocabulary tiles, ceil(V / slab_h)
     int32_t slab_h;            // slab variant: W rows per tile (a multiple of 8, <= 128)
     int32_t w_tiles;           // wide variant: vocabulary tiles of a CTA pair, ceil(V / kWideTile)
-    int32_t rows;              // wide variant: B * L, the row pitch of its partials
-    UnitPartial *partials;     // kReduce: [R][n_tiles]; wide variant: [n_tiles][rows]
+    UnitPartial *partials;     // kReduce: [R][n_tiles]
     float *logits;             // kStore: [B * L][V] fp32, written at masked rows
     uint32_t *status;          // sticky device error bits
     bool pdl;                  // host side: launch as a programmatic dependent
@@ -208,7 +207,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
 
-    // A programmatic dependent of the packing kernel: everything above overlapped its tail;
+    // A programmatic dependent of the packing kernel: everything above overlapped it;
     // the packed rows and their count are read only past this wait.
     pdl_wait();
 
@@ -763,9 +762,7 @@ constexpr int kWideMaxStages = 12;
 constexpr int kWideWarps = 12;                  // epilogue warps, three per TMEM lane quarter
 constexpr int kWideSplit = kWideWarps / 4;
 constexpr int kWideThreads = 64 + kWideWarps * 32;
-constexpr int kWideChunk = 8;                   // columns an epilogue warp turns at a time
 constexpr size_t kWideBarBytes = 512;
-constexpr int kWidePitch = kWideChunk + 1;      // both ways free of bank conflicts
 constexpr size_t kWideQuarters = (size_t)4 * kWideMaxGroup * (4 + 4 + 1);
 constexpr size_t kWideSmemBytes = 227 * 1024;
 constexpr size_t kWideFixed = kWideBarBytes + kWideQuarters;
@@ -1195,7 +1192,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                         p.S = M == -INFINITY ? 0.0f : S;
                         p.idx = I;
                         p.pad = 0;
-                        a.partials[(int64_t)(2 * n + rank) * a.rows + row0 + et] = p;
+                        a.partials[(int64_t)(row0 + et) * a.n_tiles + 2 * n + rank] = p;
                     }
                 }
             }
@@ -1213,66 +1210,81 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     tc::cluster_sync();  // no CTA leaves while its peer may still write into it
 }
 
-// One CTA: the packed list of masked rows (ascending) and its length.
-__global__ void __launch_bounds__(1024) compact_rows_kernel(const uint8_t *mask, int rows,
-                                                            int32_t *row_ids, int32_t *row_count)
+// Bytes of v that are not zero.
+__device__ __forceinline__ int count_nonzero(const uint4 &v)
 {
-    __shared__ int warp_sums[32];
-    pdl_wait();  // the mask's writer has completed
-    if (threadIdx.x == 0)
-        pdl_launch_dependents();
-    const int per = (rows + blockDim.x - 1) / blockDim.x;
-    const int lo = threadIdx.x * per;
-    const int hi = lo + per < rows ? lo + per : rows;
-    int cnt = 0;
-    for (int i = lo; i < hi; ++i)
-        cnt += mask[i] != 0;
-    // Block exclusive scan of cnt.
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o)
-            incl += y;
-    }
-    if (lane == 31)
-        warp_sums[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const int nw = blockDim.x >> 5;
-        int w = lane < nw ? warp_sums[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xFFFFFFFFu, w, o);
-            if (lane >= o)
-                w += y;
-        }
-        if (lane < nw)
-            warp_sums[lane] = w;  // inclusive over warps
-    }
-    __syncthreads();
-    int pos = incl - cnt + (warp > 0 ? warp_sums[warp - 1] : 0);
-    for (int i = lo; i < hi; ++i)
-        if (mask[i] != 0)
-            row_ids[pos++] = i;
-    if (threadIdx.x == blockDim.x - 1)
-        *row_count = pos;
+    return __popc(__vsetne4(v.x, 0u)) + __popc(__vsetne4(v.y, 0u)) + __popc(__vsetne4(v.z, 0u)) +
+           __popc(__vsetne4(v.w, 0u));
 }
 
-// CTA k copies the hidden state of packed row k (16-byte vectors).
-__global__ void gather_rows_kernel(const int4 *hidden, int64_t vec_per_row, const int32_t *row_ids,
-                                   const int32_t *row_count, int4 *packed)
+// The masked rows packed: their indices (ascending) in row_ids, their number in *row_count and
+// their hidden states, in order, in `packed` [row_count][H].  A CTA takes kPackRows neighbouring
+// rows, two warps each, and counts the masked rows before them itself (one 16-byte load per
+// thread up to 4096 rows), with the rows' own loads in flight meanwhile.  A compaction in one CTA
+// and a copy that waited for it took 1.5 us longer (fdllm_lmhead_logits on 192 rows of 50001,
+// H = 2048: 45.1 against 43.5 us).
+constexpr int kPackRows = 4;
+constexpr int kPackThreads = 64 * kPackRows;
+
+__global__ void __launch_bounds__(kPackThreads)
+    pack_rows_kernel(const uint8_t *mask, int rows, const int4 *hidden, int64_t vec_per_row,
+                     int32_t *row_ids, int32_t *row_count, int4 *packed)
 {
-    pdl_wait();  // the row list is complete
+    __shared__ int s_cnt[kPackThreads / 32];
+    pdl_wait();  // the mask's and the hidden states' writers have completed
     if (threadIdx.x == 0)
         pdl_launch_dependents();  // the GEMM may start its prologue
-    const int k = blockIdx.x;
-    if (k >= *row_count)
+    const int row0 = blockIdx.x * kPackRows;
+    const int mine = threadIdx.x >> 6, t = threadIdx.x & 63;  // this thread's row, place in it
+    bool on[kPackRows];
+#pragma unroll
+    for (int j = 0; j < kPackRows; ++j)
+        on[j] = row0 + j < rows && mask[row0 + j] != 0;
+    int cnt = 0;
+    if ((reinterpret_cast<uintptr_t>(mask) & 15u) == 0) {
+        const int whole = row0 / 16;
+        for (int i = threadIdx.x; i < whole; i += kPackThreads)
+            cnt += count_nonzero(__ldcg(reinterpret_cast<const uint4 *>(mask) + i));
+        if (threadIdx.x < row0 - whole * 16)
+            cnt += mask[whole * 16 + threadIdx.x] != 0;
+    } else {
+        for (int i = threadIdx.x; i < row0; i += kPackThreads)
+            cnt += mask[i] != 0;
+    }
+    const bool copies = mine == 0 ? on[0] : mine == 1 ? on[1] : mine == 2 ? on[2] : on[3];
+    const int4 *src = hidden + (int64_t)(row0 + mine) * vec_per_row;
+    constexpr int kAhead = 8;  // 16-byte loads in flight per thread: a row of H = 4096
+    int4 v[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i)
+        if (copies && t + 64 * i < vec_per_row)
+            v[i] = __ldg(src + t + 64 * i);
+    cnt = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)cnt);
+    if ((threadIdx.x & 31) == 0)
+        s_cnt[threadIdx.x >> 5] = cnt;
+    __syncthreads();
+    int k = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < kPackThreads / 32; ++w)
+        k += s_cnt[w];
+    total = k;
+#pragma unroll
+    for (int j = 0; j < kPackRows; ++j) {
+        total += on[j];
+        k += j < mine && on[j];
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0)
+        *row_count = total;
+    if (!copies)
         return;
-    const int4 *src = hidden + (int64_t)row_ids[k] * vec_per_row;
+    if (t == 0)
+        row_ids[k] = row0 + mine;
     int4 *dst = packed + (int64_t)k * vec_per_row;
-    for (int64_t i = threadIdx.x; i < vec_per_row; i += blockDim.x)
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i)
+        if (t + 64 * i < vec_per_row)
+            dst[t + 64 * i] = v[i];
+    for (int64_t i = t + 64 * kAhead; i < vec_per_row; i += 64)
         dst[i] = __ldg(src + i);
 }
 
@@ -1368,55 +1380,6 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
         acc = s_part[0];
         for (int w = 1; w < kCombineWarps; ++w)
             acc = fold(acc, s_part[w]);
-        store_conf(acc, row_ids[r], conf, tok);
-    }
-}
-
-// The wide variant's partials [n_tiles][rows]: a CTA takes kWideRows neighbouring rows (one
-// 64-byte segment per tile), thread t row t % 4 and tiles t / 4, t / 4 + 64, ... in order, then
-// the same symmetric folds: three butterfly steps per warp, the warps in order.
-constexpr int kWideRows = 4;
-constexpr int kWideFoldThreads = 256;
-
-__global__ void __launch_bounds__(kWideFoldThreads)
-    combine_wide_kernel(const UnitPartial *partials, int n_tiles, int rows, const int32_t *row_ids,
-                        const int32_t *row_count, float *conf, int32_t *tok)
-{
-    constexpr int kTileLanes = kWideFoldThreads / kWideRows;
-    __shared__ Part s_part[kWideFoldThreads / 32][kWideRows];
-    pdl_wait();  // every tile partial is written
-    if (threadIdx.x == 0)
-        pdl_launch_dependents();
-    const int R = *row_count;
-    const int r = blockIdx.x * kWideRows + threadIdx.x % kWideRows;
-    if (blockIdx.x * kWideRows >= R)
-        return;
-    Part acc{-__int_as_float(0x7F800000), 0.0f, kNoIdx, false};
-    constexpr int kBatch = 8;  // loads in flight per thread before the folds
-    if (r < R)
-        for (int t0 = threadIdx.x / kWideRows; t0 < n_tiles; t0 += kTileLanes * kBatch) {
-            int4 v[kBatch];
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b)
-                if (t0 + kTileLanes * b < n_tiles)
-                    v[b] = __ldcg(reinterpret_cast<const int4 *>(
-                        partials + (int64_t)(t0 + kTileLanes * b) * rows + r));
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b)
-                if (t0 + kTileLanes * b < n_tiles)
-                    acc = fold(acc, as_part(v[b]));
-        }
-#pragma unroll
-    for (int o = 16; o >= kWideRows; o >>= 1)
-        acc = fold(acc, shfl_part(acc, o));
-    const int lane = threadIdx.x & 31;
-    if (lane < kWideRows)
-        s_part[threadIdx.x >> 5][lane] = acc;
-    __syncthreads();
-    if (threadIdx.x < kWideRows && r < R) {
-        acc = s_part[0][lane];
-        for (int w = 1; w < kWideFoldThreads / 32; ++w)
-            acc = fold(acc, s_part[w][lane]);
         store_conf(acc, row_ids[r], conf, tok);
     }
 }
@@ -1766,10 +1729,12 @@ cudaError_t launch_gemm(const CUtensorMap &mh, const CUtensorMap &mw, const Gemm
     }
 }
 
-// Steps 1-3 (and 4 for the reduce epilogue) on the owned workspace.
+// Steps 1-2 (and 3 for the reduce epilogue) on the owned workspace.  The confidences and
+// argmaxes go to conf and tok [B, L], or to the workspace where those are null.
 fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, int V,
                         const uint8_t *mask, int epi, float *out_logits, cudaStream_t s,
-                        uint8_t **ws_out, LmLayout *lay_out, bool pdl = true)
+                        uint8_t **ws_out, LmLayout *lay_out, bool pdl = true,
+                        float *conf = nullptr, int32_t *tok = nullptr)
 {
     const int64_t rows = (int64_t)B * L;
     int mode = gemm_mode(rows, V);
@@ -1815,11 +1780,9 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
         return FDLLM_ERR_CUDA;
     }
 
-    if (launch_pdl(pdl, compact_rows_kernel, 1, 1024, s, mask, (int)rows, row_ids, row_count) !=
-            cudaSuccess ||
-        launch_pdl(pdl, gather_rows_kernel, (unsigned)rows, 128, s,
-                   static_cast<const int4 *>(hidden), (int64_t)(H / 8),
-                   (const int32_t *)row_ids, (const int32_t *)row_count,
+    if (launch_pdl(pdl, pack_rows_kernel, (unsigned)((rows + kPackRows - 1) / kPackRows),
+                   kPackThreads, s, mask, (int)rows, static_cast<const int4 *>(hidden),
+                   (int64_t)(H / 8), row_ids, row_count,
                    reinterpret_cast<int4 *>(packed)) != cudaSuccess)
         return FDLLM_ERR_CUDA;
     GemmArgs g;
@@ -1831,7 +1794,6 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
     g.slab_h = mode == kSlab ? bn : 0;
     g.slab_tiles = mode == kSlab ? (V + bn - 1) / bn : 0;
     g.w_tiles = w_tiles;
-    g.rows = (int)rows;
     g.partials = reinterpret_cast<UnitPartial *>(ws + lay.partials);
     g.logits = out_logits;
     g.status = reinterpret_cast<uint32_t *>(ws);
@@ -1845,36 +1807,19 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
                            : launch_gemm<kStore>(mh, mw, g, mode, bn, s);
     if (e != cudaSuccess)
         return FDLLM_ERR_CUDA;
-    if (epi == kReduce && mode == kWide) {
-        if (launch_pdl(pdl, combine_wide_kernel, (unsigned)((rows + kWideRows - 1) / kWideRows),
-                       kWideFoldThreads, s, (const UnitPartial *)g.partials, n_tiles, (int)rows,
-                       (const int32_t *)row_ids, (const int32_t *)row_count,
-                       reinterpret_cast<float *>(ws + lay.conf),
-                       reinterpret_cast<int32_t *>(ws + lay.tok)) != cudaSuccess)
-            return FDLLM_ERR_CUDA;
-    } else if (epi == kReduce) {
-        if (launch_pdl(pdl, combine_rows_kernel, (unsigned)rows, kCombineWarps * 32,
-                       s, (const UnitPartial *)g.partials, n_tiles, (const int32_t *)row_ids,
-                       (const int32_t *)row_count, reinterpret_cast<float *>(ws + lay.conf),
-                       reinterpret_cast<int32_t *>(ws + lay.tok)) != cudaSuccess)
+    if (!conf)
+        conf = reinterpret_cast<float *>(ws + lay.conf);
+    if (!tok)
+        tok = reinterpret_cast<int32_t *>(ws + lay.tok);
+    if (epi == kReduce) {
+        if (launch_pdl(pdl, combine_rows_kernel, (unsigned)rows, kCombineWarps * 32, s,
+                       (const UnitPartial *)g.partials, n_tiles, (const int32_t *)row_ids,
+                       (const int32_t *)row_count, conf, tok) != cudaSuccess)
             return FDLLM_ERR_CUDA;
     }
     *ws_out = ws;
     *lay_out = lay;
     return FDLLM_OK;
-}
-
-// Copy of the confidences and argmax of the masked rows to caller arrays.
-__global__ void scatter_conf_kernel(const float *conf, const int32_t *tok, const int32_t *row_ids,
-                                    const int32_t *row_count, float *out_conf, int32_t *out_tok)
-{
-    pdl_wait();
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= *row_count)
-        return;
-    const int row = row_ids[k];
-    out_conf[row] = conf[row];
-    out_tok[row] = tok[row];
 }
 
 }  // namespace
@@ -1943,21 +1888,10 @@ fdllm_status fdllm_lmhead_confidence(const void *hidden, const void *w_vocab, in
         return st;
     if (!out_conf || !out_argmax)
         return FDLLM_ERR_ARG;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t *ws = nullptr;
     LmLayout lay;
-    st = run_lmhead(hidden, w_vocab, B, L, H, V, mask, kReduce, nullptr, s, &ws, &lay);
-    if (st != FDLLM_OK)
-        return st;
-    const int64_t rows = (int64_t)B * L;
-    return launch_pdl(true, scatter_conf_kernel, (unsigned)((rows + 255) / 256), 256, s,
-                      reinterpret_cast<const float *>(ws + lay.conf),
-                      reinterpret_cast<const int32_t *>(ws + lay.tok),
-                      reinterpret_cast<const int32_t *>(ws + lay.row_ids),
-                      reinterpret_cast<const int32_t *>(ws + lay.row_count), out_conf,
-                      out_argmax) == cudaSuccess
-               ? FDLLM_OK
-               : FDLLM_ERR_CUDA;
+    return run_lmhead(hidden, w_vocab, B, L, H, V, mask, kReduce, nullptr,
+                      static_cast<cudaStream_t>(stream), &ws, &lay, true, out_conf, out_argmax);
 }
 
 fdllm_status fdllm_lmhead_logits(const void *hidden, const void *w_vocab, int B, int L, int H,
