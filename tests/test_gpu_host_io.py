@@ -208,3 +208,39 @@ int main(int argc, char **argv)
     assert np.array_equal(mask_out[ok], ref["mask"][ok])
     c = ref["commit"].astype(bool) & ok[:, None]
     assert np.array_equal(tok[c], ref["tokens"][c])
+
+
+@pytest.mark.parametrize("outputs", ["pinned", "pageable", "device", "mixed"])
+@pytest.mark.parametrize("where_mask", ["pinned", "pageable", "device"])
+def test_select_host_results_wherever_they_live(fd, outputs, where_mask):
+    """Page-locked result arrays are written in place by the GPU, any others are copied to: the
+    same results, tokens kept at positions not committed, the mask updated wherever it is, and a
+    batch row with unusable logits left as it was."""
+    lib = _c_select_host(fd.library_path())
+    B, L, V = 5, 70, 1024
+    g = torch.Generator().manual_seed(4)
+    x = torch.randn((B, L, V), generator=g)
+    x[2, 3, 5] = float("nan")
+    x = x.to(torch.bfloat16)
+    mask = (torch.rand((B, L), generator=g) < 0.7).to(torch.uint8) * 3
+    mask[2, 3] = 1
+    dmask = mask.cuda()
+    ref = [t.cpu() for t in fd.fdllm_select(x.cuda(), dmask, 0.5, "factor")]
+    assert fd.fdllm_device_status() == 3
+    place = {"pinned": lambda t: t.pin_memory(), "pageable": lambda t: t,
+             "device": lambda t: t.cuda()}
+    kinds = [outputs] * 3 if outputs != "mixed" else ["pinned", "pageable", "device"]
+    tok, commit, n = (place[k](t) for k, t in zip(kinds, (
+        torch.full((B, L), -7, dtype=torch.int32), torch.full((B, L), 9, dtype=torch.uint8),
+        torch.full((B,), -9, dtype=torch.int32))))
+    m = place[where_mask](mask.clone())
+    px = x.pin_memory()
+    st = lib.fdllm_select_host(px.data_ptr(), 0, B, L, V, m.data_ptr(), 0.5, 1, tok.data_ptr(),
+                               commit.data_ptr(), n.data_ptr(),
+                               torch.cuda.current_stream().cuda_stream)
+    assert st == 0 and fd.fdllm_device_status() == 3
+    tok, commit, n, m = (t.cpu() for t in (tok, commit, n, m))
+    on = commit != 0
+    assert torch.equal(n, ref[2]) and n[2] == -1 and torch.equal(commit, ref[1])
+    assert torch.equal(m, dmask.cpu()) and torch.equal(m[2], mask[2])
+    assert torch.equal(tok[on], ref[0][on]) and (tok[~on] == -7).all()
