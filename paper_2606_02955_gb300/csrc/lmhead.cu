@@ -94,7 +94,8 @@ struct GemmArgs {
     int32_t k_blocks;          // ceil(H / BK)
     int32_t slab_tiles;        // slab variant: vocabulary tiles, ceil(V / slab_h)
     int32_t slab_h;            // slab variant: W rows per tile (a multiple of 8, <= 128)
-    int32_t w_tiles;           // wide variant: vocabulary tiles of a CTA pair, ceil(V / kWideTile)
+    int32_t wide_h;            // wide variant: W rows per CTA and tile (a multiple of 8, <= 128)
+    int32_t w_tiles;           // wide variant: vocabulary tiles of a CTA pair, ceil(V / 2 wide_h)
     UnitPartial *partials;     // kReduce: [R][n_tiles]
     float *logits;             // kStore: [B * L][V] fp32, written at masked rows
     uint32_t *status;          // sticky device error bits
@@ -743,8 +744,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // ----------------------------------------------------------------------------- wide variant
-// W is the M = 256 operand of a CTA pair (a tile of 256 vocabulary entries, 128 per CTA, lane =
-// entry) and the packed rows are N, in blocks of up to 256 rows (one MMA group, two accumulators
+// W is the M = 256 operand of a CTA pair (a tile of 2 h vocabulary entries, h <= 128 per CTA, lane
+// = entry, see wide_height) and the packed rows are N, in blocks of up to 256 rows (one MMA group, two accumulators
 // in turn) or, for 257 to 320 rows, one block of two groups that share every W stage (three
 // accumulators).  What bounds the solo variant at 2 to 6 row tiles is the 64 B/clock at which an
 // SM receives from L2: its stage is 42 KB for 416 MMA cycles (101 B/clock wanted, 65 measured).
@@ -755,7 +756,6 @@ __global__ void __launch_bounds__(kThreads, 1)
 // 410, 32 426 against 422 and 64 795 against 785 (pair): the host takes it up to 28 x 32 rows.
 // Other cuts measured: 288 rows in two blocks 220, 381 rows in one block of two groups 245, 480
 // rows in one block 311 against 293 in two.
-constexpr int kWideTile = 256;                  // vocabulary entries per CTA pair and item
 constexpr int kWideMaxGroup = 256;              // MMA columns per group
 constexpr int kWideTwoGroups = 320;             // rows that still make one block, of two groups
 constexpr int kWideMaxStages = 12;
@@ -962,8 +962,10 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     const int R = __shfl_sync(0xFFFFFFFFu, *a.row_count, 0);
     const WideCut cut = wide_cut(R);
     const int block_rows = cut.groups * cut.g;
+    const int h = a.wide_h;
     const uint32_t half_bytes = (uint32_t)(cut.g / 2 * BK * 2);  // a CTA's share of a group's stage
-    const uint32_t stage_bytes = kABytes + cut.groups * half_bytes;
+    const uint32_t a_bytes = (uint32_t)(h * BK * 2);
+    const uint32_t stage_bytes = a_bytes + cut.groups * half_bytes;
     const int stages = min(kWideMaxStages, (int)(ring_bytes / stage_bytes));
     const WideItems items(cut, a.w_tiles, (int)tc::cluster_count_x(), (int)tc::cluster_id_x());
 
@@ -982,8 +984,8 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                 break;
             const int n = t / cut.n_blocks;
             const int row0 = t % cut.n_blocks * block_rows + rank * (cut.g / 2);
-            const int w_row = n * kWideTile + rank * BM;
-            const uint32_t bytes = kABytes + (uint32_t)(j1 - j0) * half_bytes;
+            const int w_row = (2 * n + rank) * h;
+            const uint32_t bytes = a_bytes + (uint32_t)(j1 - j0) * half_bytes;
             for (int kb = 0; kb < a.k_blocks; ++kb) {
                 if (!warp_wait(&empty[s], ph ^ 1u, a.status, abort_flag)) {
                     ok = false;
@@ -996,9 +998,9 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                     const uint32_t bar0 = tc::map_to_rank(&full[s], 0);
                     uint8_t *stage = smem + s * stage_bytes;
                     tc::tma_load_2d_pair_hint(stage, &map_w, kb * BK, w_row, bar0, pol);
-                    tc::tma_load_2d_pair(stage + kABytes, map_h, kb * BK, row0 + j0 * cut.g, bar0);
+                    tc::tma_load_2d_pair(stage + a_bytes, map_h, kb * BK, row0 + j0 * cut.g, bar0);
                     if (j1 - j0 == 2)
-                        tc::tma_load_2d_pair(stage + kABytes + half_bytes, map_h, kb * BK,
+                        tc::tma_load_2d_pair(stage + a_bytes + half_bytes, map_h, kb * BK,
                                              row0 + cut.g, bar0);
                 }
                 filled = min(filled + 1, (uint32_t)stages);
@@ -1045,7 +1047,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                         }
                         tc::fence_after_sync();
                         const uint64_t ad = tc::sw128_kmajor_desc(smem + s * stage_bytes);
-                        const uint64_t bd = ad + (kABytes >> 4);
+                        const uint64_t bd = ad + (a_bytes >> 4);
                         if (elect_one()) {
 #pragma unroll
                             for (int k = 0; k < BK / 16; ++k)
@@ -1080,7 +1082,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                         }
                     }
                     const uint64_t ad = tc::sw128_kmajor_desc(smem + s1 * stage_bytes);
-                    const uint64_t bd = ad + (kABytes >> 4) + (half_bytes >> 4);
+                    const uint64_t bd = ad + (a_bytes >> 4) + (half_bytes >> 4);
                     if (elect_one()) {
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k)
@@ -1120,7 +1122,8 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                 break;
             const int n = t / cut.n_blocks;
             const int blk0 = t % cut.n_blocks * block_rows;
-            const int ent0 = n * kWideTile + rank * BM;
+            const int ent0 = (2 * n + rank) * h;  // this CTA's entries: ent0 .. ends - 1
+            const int ends = min(a.V, ent0 + h);
             for (int j = j0; j < j1; ++j, ++used) {
                 const uint32_t buf = used % cut.buffers, turn = used / cut.buffers;
                 const bool got = wait_or_abort(&tfull[buf], turn & 1u, a.status, abort_flag);
@@ -1154,13 +1157,13 @@ __global__ void __launch_bounds__(kWideThreads, 1)
 #pragma unroll
                         for (int k = 0; k < 32; ++k) {
                             const int64_t row = __shfl_sync(0xFFFFFFFFu, mine, k);
-                            if (c + k < live && ent < a.V)
+                            if (c + k < live && ent < ends)
                                 a.logits[row * a.V + ent] = x[k / 16][k % 16];
                         }
                     } else {
                         float M, S;
                         uint32_t I;
-                        wide_reduce_block(x, a.V - (ent0 + quarter * 32), lane, M, S, I);
+                        wide_reduce_block(x, ends - (ent0 + quarter * 32), lane, M, S, I);
                         const int at = quarter * kWideMaxGroup + c + wide_column(lane);
                         q_M[at] = M;
                         q_S[at] = S;
@@ -1505,6 +1508,20 @@ int slab_height(int V)
     return best;
 }
 
+// The wide variant's W rows per CTA and tile.  A few rows leave it bound by W alone, and the slab
+// variant's heights (104 for LLaDA's V: eight whole rounds instead of six and a half) balance
+// that: of 128 rows 8 masked 155 against 163 us, 32 157 against 163, 96 158 against 159, 128 160
+// against 160.  More rows make it the tensor cores', whose M = 256 a lower tile leaves partly
+// unused: of 192 rows all masked 167 against 164, of 256 190 against 178 (but 16 of them 157
+// against 163), 288 of 384 229 against 195.  So the line lies at 192, by the shape alone: a row's
+// partials must not depend on how many rows are masked.
+constexpr int kWideLowRows = 192;
+
+int wide_height(int64_t rows, int V)
+{
+    return rows <= kWideLowRows ? slab_height(V) : BM;
+}
+
 // The slab variant's grid: one CTA per SM, or one per tile if there are fewer.
 int slab_grid(int V)
 {
@@ -1738,15 +1755,15 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
 {
     const int64_t rows = (int64_t)B * L;
     int mode = gemm_mode(rows, V);
-    int bn = 0, n_tiles = 0;
-    const int w_tiles = (V + kWideTile - 1) / kWideTile;
+    int bn = 0, n_tiles = 0, w_tiles = 0;
     LmLayout lay;
     // partials per row: one per vocabulary tile (per CTA of the pair in the wide variant), or
     // one per CTA of the slab variant
     auto plan = [&] {
         bn = mode == kSlab   ? slab_height(V)
-             : mode == kWide ? kWideTile / 2
+             : mode == kWide ? wide_height(rows, V)
                              : choose_bn(rows, V, mode == kPair);
+        w_tiles = (V + 2 * bn - 1) / (2 * bn);
         n_tiles = mode == kSlab   ? slab_grid(V)
                   : mode == kWide ? 2 * w_tiles
                                   : (V + bn - 1) / bn;
@@ -1794,6 +1811,7 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
     g.slab_h = mode == kSlab ? bn : 0;
     g.slab_tiles = mode == kSlab ? (V + bn - 1) / bn : 0;
     g.w_tiles = w_tiles;
+    g.wide_h = mode == kWide ? bn : 0;
     g.partials = reinterpret_cast<UnitPartial *>(ws + lay.partials);
     g.logits = out_logits;
     g.status = reinterpret_cast<uint32_t *>(ws);

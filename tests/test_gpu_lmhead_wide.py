@@ -16,7 +16,10 @@ pytestmark = pytest.mark.gpu
 # (B, L, H, V, masked rows)
 SHAPES = [
     (1, 3, 72, 40, 2),           # V within the even CTA's half of one tile
-    (2, 20, 64, 129, 33),        # one entry in the odd CTA's half; one K-block
+    (2, 20, 64, 129, 33),        # few entries in the odd CTA's half; one K-block
+    (2, 40, 192, 34048, 70),     # tiles of 2 x 112 entries
+    (3, 64, 72, 36480, 150),     # of 2 x 120, at the most rows that take low tiles
+    (5, 32, 64, 9750, 160),      # of 2 x 96, the last one ragged
     (4, 64, 128, 300, 193),      # a group of 224: two passes over its columns
     (4, 64, 128, 300, 256),      # one group of 256: two accumulators
     (4, 65, 192, 5000, 257),     # two groups; all 20 tiles split between two pairs
