@@ -8,7 +8,8 @@
 // Launch sequence on one stream (all rows of one step), chained by programmatic dependent
 // launches:
 //   1. pack_rows_kernel      the masked rows' indices, their count and their hidden states,
-//                            packed [R, H] (TMA-friendly)
+//                            packed [R, H] (TMA-friendly); two kernels, compact_rows and
+//                            gather_rows, before the pair GEMM
 //   2. lmhead_gemm_kernel    persistent tcgen05 GEMM: warp 0 issues TMA loads into a ring of
 //                            stages, warp 1 issues tcgen05.mma into one of two TMEM
 //                            accumulators, warps 2-5 reduce (or store) the other one; solo
@@ -87,7 +88,7 @@ struct TileCfg {
 };
 
 struct GemmArgs {
-    const int32_t *row_count;  // R, written by pack_rows_kernel
+    const int32_t *row_count;  // R, written by the packing
     const int32_t *row_ids;    // [R] global row (b * L + l) of each packed row
     int32_t V;
     int32_t n_tiles;           // partials per row: ceil(V / BN), or the slab variant's grid
@@ -1291,6 +1292,75 @@ __global__ void __launch_bounds__(kPackThreads)
         dst[i] = __ldg(src + i);
 }
 
+// The pair variant's rows are packed by two kernels, this list and a copy by one small CTA per row,
+// although that takes 2 us longer: the GEMM's clusters are then placed while 2048 such CTAs come
+// and go, mostly one die of the GPU first, and the six pairs that share a W tile mostly share its
+// L2.  Behind pack_rows_kernel they end up mixed, which costs more than 2 us of the power that
+// limits this variant: 64 x 32 rows back to back 891 against 902 us (clusters in SM order 903).
+//
+// One CTA: the packed list of masked rows (ascending) and its length.
+__global__ void __launch_bounds__(1024) compact_rows_kernel(const uint8_t *mask, int rows,
+                                                            int32_t *row_ids, int32_t *row_count)
+{
+    __shared__ int warp_sums[32];
+    pdl_wait();  // the mask's writer has completed
+    if (threadIdx.x == 0)
+        pdl_launch_dependents();
+    const int per = (rows + blockDim.x - 1) / blockDim.x;
+    const int lo = threadIdx.x * per;
+    const int hi = lo + per < rows ? lo + per : rows;
+    int cnt = 0;
+    for (int i = lo; i < hi; ++i)
+        cnt += mask[i] != 0;
+    // Block exclusive scan of cnt.
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o)
+            incl += y;
+    }
+    if (lane == 31)
+        warp_sums[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        const int nw = blockDim.x >> 5;
+        int w = lane < nw ? warp_sums[lane] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, w, o);
+            if (lane >= o)
+                w += y;
+        }
+        if (lane < nw)
+            warp_sums[lane] = w;  // inclusive over warps
+    }
+    __syncthreads();
+    int pos = incl - cnt + (warp > 0 ? warp_sums[warp - 1] : 0);
+    for (int i = lo; i < hi; ++i)
+        if (mask[i] != 0)
+            row_ids[pos++] = i;
+    if (threadIdx.x == blockDim.x - 1)
+        *row_count = pos;
+}
+
+// CTA k copies the hidden state of packed row k (16-byte vectors).
+__global__ void gather_rows_kernel(const int4 *hidden, int64_t vec_per_row, const int32_t *row_ids,
+                                   const int32_t *row_count, int4 *packed)
+{
+    pdl_wait();  // the row list is complete
+    if (threadIdx.x == 0)
+        pdl_launch_dependents();  // the GEMM may start its prologue
+    const int k = blockIdx.x;
+    if (k >= *row_count)
+        return;
+    const int4 *src = hidden + (int64_t)row_ids[k] * vec_per_row;
+    int4 *dst = packed + (int64_t)k * vec_per_row;
+    for (int64_t i = threadIdx.x; i < vec_per_row; i += blockDim.x)
+        dst[i] = __ldg(src + i);
+}
+
 struct Part {
     float M, S;
     uint32_t idx;
@@ -1797,11 +1867,20 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
         return FDLLM_ERR_CUDA;
     }
 
-    if (launch_pdl(pdl, pack_rows_kernel, (unsigned)((rows + kPackRows - 1) / kPackRows),
-                   kPackThreads, s, mask, (int)rows, static_cast<const int4 *>(hidden),
-                   (int64_t)(H / 8), row_ids, row_count,
-                   reinterpret_cast<int4 *>(packed)) != cudaSuccess)
+    if (mode == kPair) {
+        if (launch_pdl(pdl, compact_rows_kernel, 1, 1024, s, mask, (int)rows, row_ids,
+                       row_count) != cudaSuccess ||
+            launch_pdl(pdl, gather_rows_kernel, (unsigned)rows, 128, s,
+                       static_cast<const int4 *>(hidden), (int64_t)(H / 8),
+                       (const int32_t *)row_ids, (const int32_t *)row_count,
+                       reinterpret_cast<int4 *>(packed)) != cudaSuccess)
+            return FDLLM_ERR_CUDA;
+    } else if (launch_pdl(pdl, pack_rows_kernel, (unsigned)((rows + kPackRows - 1) / kPackRows),
+                          kPackThreads, s, mask, (int)rows, static_cast<const int4 *>(hidden),
+                          (int64_t)(H / 8), row_ids, row_count,
+                          reinterpret_cast<int4 *>(packed)) != cudaSuccess) {
         return FDLLM_ERR_CUDA;
+    }
     GemmArgs g;
     g.row_count = row_count;
     g.row_ids = row_ids;
