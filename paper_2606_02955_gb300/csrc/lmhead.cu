@@ -753,10 +753,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Here a stage is (128 + N / 2) x 128 B for 2 N cycles: 75 B/clock at N = 192, 58 at 320, and no
 // row tile is padded to 128.  LLaDA's head, 3/4 of B x 32 rows, whole fdllm_lmhead_confidence
 // pass, this variant against the better of solo and pair: B = 3 (72 rows) 160 against 163 us,
-// 8 170 against 190, 12 204 against 251, 16 244 against 261, 24 346 against 396, 28 385 against
+// 8 165 against 190, 12 194 against 251, 16 244 against 261, 24 346 against 396, 28 385 against
 // 410, 32 426 against 422 and 64 795 against 785 (pair): the host takes it up to 28 x 32 rows.
-// Other cuts measured: 288 rows in two blocks 220, 381 rows in one block of two groups 245, 480
-// rows in one block 311 against 293 in two.
+// Other cuts measured: 288 rows in two blocks 220, in two groups of 160 instead of 160 and 128
+// 200 (back to back, at the power limit, 235 against 225), 381 rows in one block of two groups
+// 245, 480 rows in one block 311 against 293 in two.
 constexpr int kWideMaxGroup = 256;              // MMA columns per group
 constexpr int kWideTwoGroups = 320;             // rows that still make one block, of two groups
 constexpr int kWideMaxStages = 12;
@@ -776,11 +777,13 @@ struct WideRowMaps {
     CUtensorMap m[kWideMaps];
 };
 
-// How R rows are cut: n_blocks blocks of `groups` groups of g rows each, g a multiple of 32 (what
-// lies past R is padding), items (W tile, block) with the block fastest, so that the pairs
-// sharing a W tile work on it at the same time.  `buffers` accumulators of g columns take turns.
+// How R rows are cut: n_blocks blocks of g rows, or one block of two groups of g and g1 rows, both
+// multiples of 32 (what lies past R is padding), items (W tile, block) with the block fastest, so
+// that the pairs sharing a W tile work on it at the same time.  `buffers` accumulators of g
+// columns take turns.
 struct WideCut {
-    int n_blocks, groups, g, buffers;
+    int n_blocks, groups, g, g1, buffers;
+    __device__ __forceinline__ int width(int j) const { return j == 0 ? g : g1; }
 };
 
 __device__ __forceinline__ WideCut wide_cut(int R)
@@ -790,6 +793,7 @@ __device__ __forceinline__ WideCut wide_cut(int R)
     const int per = c.n_blocks > 0 ? (R + c.n_blocks - 1) / c.n_blocks : 1;
     c.groups = per > kWideMaxGroup ? 2 : 1;
     c.g = ((per + c.groups - 1) / c.groups + 31) / 32 * 32;
+    c.g1 = c.groups == 2 ? (per - c.g + 31) / 32 * 32 : 0;
     c.buffers = min(4, (int)kTmemCols / c.g);
     return c;
 }
@@ -962,11 +966,12 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     const int rank = (int)tc::cluster_ctarank();
     const int R = __shfl_sync(0xFFFFFFFFu, *a.row_count, 0);
     const WideCut cut = wide_cut(R);
-    const int block_rows = cut.groups * cut.g;
+    const int block_rows = cut.g;  // one block where there are two groups
     const int h = a.wide_h;
-    const uint32_t half_bytes = (uint32_t)(cut.g / 2 * BK * 2);  // a CTA's share of a group's stage
+    // a CTA's share of a group of g rows in a stage
+    auto half_bytes = [](int g) { return (uint32_t)(g / 2 * BK * 2); };
     const uint32_t a_bytes = (uint32_t)(h * BK * 2);
-    const uint32_t stage_bytes = a_bytes + cut.groups * half_bytes;
+    const uint32_t stage_bytes = a_bytes + half_bytes(cut.g) + half_bytes(cut.g1);
     const int stages = min(kWideMaxStages, (int)(ring_bytes / stage_bytes));
     const WideItems items(cut, a.w_tiles, (int)tc::cluster_count_x(), (int)tc::cluster_id_x());
 
@@ -974,7 +979,6 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     // stay warp-uniform, which the issuing instructions need them to be.
     if (warp == 0) {
         const uint64_t pol = make_evict_first_policy();  // W is read once (per row block)
-        const CUtensorMap *map_h = &maps_h.m[cut.g / 32 - 1];
         int s = 0;
         uint32_t ph = 0, filled = 0;
         bool ok = true;
@@ -984,9 +988,14 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             if (t < 0)
                 break;
             const int n = t / cut.n_blocks;
-            const int row0 = t % cut.n_blocks * block_rows + rank * (cut.g / 2);
+            const int g = cut.width(j0);
+            const int row0 = t % cut.n_blocks * block_rows + j0 * cut.g + rank * (g / 2);
+            const int row1 = cut.g + rank * (cut.g1 / 2);  // the second of two groups
+            const CUtensorMap *map0 = &maps_h.m[g / 32 - 1];
+            const CUtensorMap *map1 = &maps_h.m[j1 - j0 == 2 ? cut.g1 / 32 - 1 : 0];
             const int w_row = (2 * n + rank) * h;
-            const uint32_t bytes = a_bytes + (uint32_t)(j1 - j0) * half_bytes;
+            const uint32_t bytes =
+                a_bytes + half_bytes(g) + (j1 - j0 == 2 ? half_bytes(cut.g1) : 0u);
             for (int kb = 0; kb < a.k_blocks; ++kb) {
                 if (!warp_wait(&empty[s], ph ^ 1u, a.status, abort_flag)) {
                     ok = false;
@@ -999,10 +1008,10 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                     const uint32_t bar0 = tc::map_to_rank(&full[s], 0);
                     uint8_t *stage = smem + s * stage_bytes;
                     tc::tma_load_2d_pair_hint(stage, &map_w, kb * BK, w_row, bar0, pol);
-                    tc::tma_load_2d_pair(stage + a_bytes, map_h, kb * BK, row0 + j0 * cut.g, bar0);
+                    tc::tma_load_2d_pair(stage + a_bytes, map0, kb * BK, row0, bar0);
                     if (j1 - j0 == 2)
-                        tc::tma_load_2d_pair(stage + a_bytes + half_bytes, map_h, kb * BK,
-                                             row0 + cut.g, bar0);
+                        tc::tma_load_2d_pair(stage + a_bytes + half_bytes(g), map1, kb * BK, row1,
+                                             bar0);
                 }
                 filled = min(filled + 1, (uint32_t)stages);
                 if (++s == stages) {
@@ -1018,7 +1027,6 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         __syncwarp();
     } else if (warp == 1) {
         if (rank == 0) {
-            const uint32_t idesc = tc::idesc_bf16_f32(2 * BM, cut.g);
             int s = 0;
             uint32_t ph = 0;
             uint32_t used = 0;  // groups accumulated so far
@@ -1035,6 +1043,8 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                     break;
                 tc::fence_after_sync();
                 const uint32_t d0 = tmem_base + b0 * cut.g, d1 = tmem_base + b1 * cut.g;
+                const uint32_t idesc0 = tc::idesc_bf16_f32(2 * BM, cut.width(j0));
+                const uint32_t idesc1 = tc::idesc_bf16_f32(2 * BM, cut.g1);
                 // Two groups share each stage.  While the second group's accumulator is still
                 // being read, the first one runs ahead over the stages of the ring (k0, at s);
                 // the second one follows (k1, at s1), the last to read a stage.
@@ -1052,7 +1062,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                         if (elect_one()) {
 #pragma unroll
                             for (int k = 0; k < BK / 16; ++k)
-                                tc::mma_bf16_pair(d0, ad + 2u * k, bd + 2u * k, idesc,
+                                tc::mma_bf16_pair(d0, ad + 2u * k, bd + 2u * k, idesc0,
                                                   (k0 | k) != 0);
                             if (!two)
                                 tc::commit_pair_multicast(&empty[s]);
@@ -1083,11 +1093,11 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                         }
                     }
                     const uint64_t ad = tc::sw128_kmajor_desc(smem + s1 * stage_bytes);
-                    const uint64_t bd = ad + (a_bytes >> 4) + (half_bytes >> 4);
+                    const uint64_t bd = ad + (a_bytes >> 4) + (half_bytes(cut.g) >> 4);
                     if (elect_one()) {
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k)
-                            tc::mma_bf16_pair(d1, ad + 2u * k, bd + 2u * k, idesc, (k1 | k) != 0);
+                            tc::mma_bf16_pair(d1, ad + 2u * k, bd + 2u * k, idesc1, (k1 | k) != 0);
                         tc::commit_pair_multicast(&empty[s1]);
                     }
                     ++k1;
@@ -1138,7 +1148,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                 const uint32_t taddr =
                     tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * cut.g;
                 const int row0 = blk0 + j * cut.g;
-                const int live = min(cut.g, R - row0);  // columns that are rows
+                const int live = min(cut.width(j), R - row0);  // columns that are rows
 #pragma unroll 1
                 for (int c = third * 32; c < live; c += kWideSplit * 32) {
                     float x[2][16];

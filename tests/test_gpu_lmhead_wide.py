@@ -23,7 +23,8 @@ SHAPES = [
     (4, 64, 128, 300, 193),      # a group of 224: two passes over its columns
     (4, 64, 128, 300, 256),      # one group of 256: two accumulators
     (4, 65, 192, 5000, 257),     # two groups; all 20 tiles split between two pairs
-    (10, 32, 256, 12000, 288),   # 47 tiles: no split, a round of its own
+    (10, 32, 256, 12000, 288),   # groups of 160 and 128; 47 tiles: no split, a round of its own
+    (10, 32, 64, 25000, 288),    # the same, the last round split between the groups
     (5, 64, 128, 25000, 320),    # 98 tiles: a whole round, then a split one
     (6, 64, 136, 700, 321),      # two blocks of one group; a ragged K tail
     (9, 60, 64, 1000, 513),      # three blocks
