@@ -229,12 +229,15 @@ fdllm_status fdllm_gather_masked_rows(const void *src, void *dst, int dtype, int
  *   mask, out_tokens, out_commit, out_n  host (or device) arrays of fdllm_select's shapes;
  *           mask is updated in place and out_tokens keeps its values at positions not
  *           committed, as in fdllm_select.
- * The library copies mask and out_tokens to a device staging buffer of its own (per device,
- * grown on demand with cudaMalloc, released by fdllm_release_workspace), runs the step on
- * `stream` with the library workspace, copies out_tokens, out_commit, out_n and the mask
- * back and synchronises `stream` before it returns: the results are in place when the call
- * returns.  Argument errors are reported before anything is enqueued; the same device
- * errors as fdllm_select (fdllm_device_status).  Not for stream capture (it synchronises).
+ * The library copies the mask to a device staging buffer of its own (per device, grown on
+ * demand with cudaMalloc, released by fdllm_release_workspace), runs the step on `stream`
+ * with the library workspace and synchronises `stream` before it returns: the results are in
+ * place when the call returns.  Where out_tokens, out_commit and out_n are page-locked and
+ * the mask is in host memory, the step writes the three over the host link and the host
+ * clears the committed positions of the mask after the synchronisation; otherwise out_tokens
+ * is staged as well, and all four are copied back.  Argument errors are reported before
+ * anything is enqueued; the same device errors as fdllm_select (fdllm_device_status).  Not
+ * for stream capture (it synchronises).
  * Calls share the staging buffer and the library workspace of their device: calls from
  * several host threads at once must be serialised by the caller.  The paper has no
  * counterpart. */

@@ -4,6 +4,7 @@
 // the step and the copies of its results back to the host in one call.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <mutex>
 
@@ -13,10 +14,19 @@
 namespace fdllm {
 namespace {
 
-// One CTA per (b, l) row: copies the row's 16-byte vectors when the position is masked.
-__global__ void __launch_bounds__(256) gather_masked_rows_kernel(const int4 *src, int4 *dst,
-                                                                 const uint8_t *mask,
-                                                                 int64_t vec_per_row)
+// Bound by the host link (210 GB/s), which takes about 0.4 MB in flight to fill: with few rows a
+// row is cut into parts of at least 16 KB (one round of a CTA's loads), so that a few masked rows
+// fill it too.  One CTA per row against parts, fdllm_select_host on 32 positions of LLaDA's
+// vocabulary: 5 % masked 43.5 -> 36 us, 15 % 47.5 -> 39.8, 50 % 52.2 -> 46.5.  The most CTAs: at
+// 8 x 32 positions, 4 parts a row (8 CTAs per SM) took 197 us, one part 195.4.
+constexpr int64_t kGatherPartVecs = 1024;
+constexpr int64_t kGatherCtas = 2 * 152;
+
+// Copies the 16-byte vectors of the masked (b, l) rows: row blockIdx.x, the part_vecs vectors of
+// part blockIdx.y.
+__global__ void __launch_bounds__(256)
+    gather_masked_rows_kernel(const int4 *src, int4 *dst, const uint8_t *mask,
+                              int64_t vec_per_row, int64_t part_vecs)
 {
     pdl_wait();  // the mask's writer has completed
     if (threadIdx.x == 0)
@@ -24,18 +34,20 @@ __global__ void __launch_bounds__(256) gather_masked_rows_kernel(const int4 *src
     const int64_t row = blockIdx.x;
     if (mask[row] == 0)
         return;
-    const int4 *s = src + row * vec_per_row;
-    int4 *d = dst + row * vec_per_row;
+    const int64_t begin = blockIdx.y * part_vecs;
+    const int64_t n = min(part_vecs, vec_per_row - begin);
+    const int4 *s = src + row * vec_per_row + begin;
+    int4 *d = dst + row * vec_per_row + begin;
     int64_t i = threadIdx.x;
     // Four loads in flight per thread: each crosses the host link with its full latency.
-    for (; i + 3 * 256 < vec_per_row; i += 4 * 256) {
+    for (; i + 3 * 256 < n; i += 4 * 256) {
         const int4 a = s[i], b = s[i + 256], c = s[i + 512], e = s[i + 768];
         d[i] = a;
         d[i + 256] = b;
         d[i + 512] = c;
         d[i + 768] = e;
     }
-    for (; i < vec_per_row; i += 256)
+    for (; i < n; i += 256)
         d[i] = s[i];
 }
 
@@ -86,8 +98,12 @@ bool on_host(const void *p)
 cudaError_t launch_gather(const void *dsrc, void *dst, const uint8_t *mask, int64_t rows,
                           int64_t row_bytes, cudaStream_t stream)
 {
+    const int64_t vecs = row_bytes / 16;
+    const int64_t most = std::max<int64_t>(1, kGatherCtas / rows);
+    const int64_t want = std::min((vecs + kGatherPartVecs - 1) / kGatherPartVecs, most);
+    const int64_t part_vecs = (vecs + want - 1) / want;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)rows);
+    cfg.gridDim = dim3((unsigned)rows, (unsigned)((vecs + part_vecs - 1) / part_vecs));
     cfg.blockDim = dim3(256);
     cfg.stream = stream;
     cudaLaunchAttribute a[1];
@@ -96,7 +112,7 @@ cudaError_t launch_gather(const void *dsrc, void *dst, const uint8_t *mask, int6
     cfg.attrs = a;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, gather_masked_rows_kernel, static_cast<const int4 *>(dsrc),
-                              static_cast<int4 *>(dst), mask, row_bytes / 16);
+                              static_cast<int4 *>(dst), mask, vecs, part_vecs);
 }
 
 // fdllm_select_host's device staging, one buffer per device, grown on demand (allocated

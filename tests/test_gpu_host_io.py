@@ -24,6 +24,23 @@ def test_gather_from_pinned_host_copies_masked_rows_only(fd, name):
     assert (got[~mk] == 3.0).all()
 
 
+@pytest.mark.parametrize("B, L, vecs", [
+    (1, 1, 1), (1, 1, 1024), (1, 1, 1025), (1, 2, 3 * 1024 + 5), (1, 1, 304 * 1024 + 7),
+    (19, 8, 2049), (38, 8, 1025), (305, 1, 1025)])
+def test_gather_parts_of_a_row(fd, B, L, vecs):
+    """Rows cut into parts: one vector, one part, one vector more, remainders, more vectors
+    than the most parts hold, two parts (152 rows), one (304) and no room for one a row (305)."""
+    x = torch.randint(-2 ** 31, 2 ** 31, (B, L, 4 * vecs), dtype=torch.int32).view(torch.float32)
+    mask = (torch.rand(B, L) < 0.5).to(torch.uint8)
+    mask[-1, -1] = 1
+    dst = torch.full(x.shape, 3.0, device="cuda")
+    fd.fdllm_gather_masked_rows(x.pin_memory(), mask.cuda(), dst)
+    torch.cuda.synchronize()
+    got, mk = dst.cpu(), mask.bool()
+    assert torch.equal(got[mk].view(torch.int32), x[mk].view(torch.int32))
+    assert (got[~mk] == 3.0).all()
+
+
 def test_gather_from_device_and_rejects_pageable(fd):
     x = torch.randn(2, 8, 512, device="cuda").to(torch.bfloat16)
     mask = torch.tensor([[1, 0] * 4, [0, 1] * 4], dtype=torch.uint8, device="cuda")
