@@ -181,6 +181,7 @@ fdllm_status run_select(const void *logits, int dtype, int B, int L, int V, uint
         return FDLLM_ERR_CUDA;
     ProfileSelectArgs pa;
     pa.units_per_row = ra.units_per_row;
+    pa.warp_units = ra.warp_units;
     pa.partials = ra.partials;
     pa.next_unit = ra.next_unit;
     pa.conf = nullptr;
@@ -411,6 +412,7 @@ fdllm_status fdllm_confidence(const void *logits, int dtype, int B, int L, int V
     fa.out_conf = out_conf;
     fa.out_tok = out_argmax;
     fa.next_unit = ra.next_unit;
+    fa.warp_units = ra.warp_units;
     if (launch_finalize(fa, s) != cudaSuccess)
         return FDLLM_ERR_CUDA;
     return FDLLM_OK;

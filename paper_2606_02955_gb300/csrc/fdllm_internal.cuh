@@ -129,6 +129,7 @@ struct FinalizeArgs {
     float *out_conf;
     int32_t *out_tok;
     uint32_t *next_unit;
+    bool warp_units;  // the partials come from warp units
 };
 
 cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t stream);
@@ -159,6 +160,7 @@ struct ProfileSelectArgs {
     uint32_t *status;        // nullable: the timeout bit set -> every row reports a device
                              // error; a non-finite row sets the non-finite bit
     bool pdl = true;         // with partials: launch as a programmatic dependent
+    bool warp_units = false; // the partials come from warp units
 };
 
 cudaError_t launch_profile_select(const ProfileSelectArgs &a, cudaStream_t stream);

@@ -52,6 +52,13 @@ __device__ __forceinline__ float key_conf(uint64_t key)
     return __uint_as_float(kOneBits - (uint32_t)(key >> 32));
 }
 
+// Barrier of a row's W warps (the CTA may hold idle ones, see kSpreadThreads).
+template <int W>
+__device__ __forceinline__ void row_barrier()
+{
+    asm volatile("barrier.cta.sync 1, %0;" ::"n"(32 * W) : "memory");
+}
+
 // A row of more than 32 positions is held by W warps of K keys per thread: element
 // (w K + r) 32 + lane is key[r] of that lane of warp w.
 //
@@ -84,7 +91,7 @@ __device__ __forceinline__ void sort_keys(uint64_t (&key)[K], uint64_t *buf)
 #pragma unroll
                 for (int r = 0; r < K; ++r)
                     buf[turn + idx0 + 32 * r] = key[r];
-                __syncthreads();
+                row_barrier<W>();
 #pragma unroll
                 for (int r = 0; r < K; ++r) {
                     const uint64_t other = buf[turn + ((idx0 + 32 * r) ^ j)];
@@ -136,7 +143,7 @@ __device__ __forceinline__ void scan_elements(V (&v)[K], V *warp_tot)
             total += __shfl_sync(0xFFFFFFFFu, v[r], 31);
         if (lane == 0)
             warp_tot[w] = total;
-        __syncthreads();
+        row_barrier<W>();
         for (int i = 0; i < w; ++i)
             base += warp_tot[i];
     }
@@ -164,10 +171,30 @@ __device__ __forceinline__ bool rule_accepts(int mode, int n, float cn, int64_t 
     return cn >= tau_f;  // threshold: c_(n) >= tau
 }
 
+// Where rows' CTAs start while the kernel before them holds the SMs (the warp units all registers of
+// every SM, the confidences' own pass many of its threads), small ones are all placed on the first
+// few SMs to be freed, where their loads and sorts then queue.  CTAs of 512 threads, the warps
+// beyond a row's own returning at once, spread over more.  Time over the reduction alone, a row's
+// own warps against 512 threads: 64 x 32 positions of 32000 bf16 logits 7.8 -> 3.1 us, of 20000 5.0
+// -> 2.6, 131 x 61 of 20008 fp16 7.5 -> 5.1, 64 x 256 of 16384 8.1 -> 4.9 (with 256 threads 3.2,
+// 2.4, 5.1 and 7.0; with 1024 3.2, 2.4, 6.2 and 6.4).  After CTA units, which leave room for small
+// CTAs beside them, it gains nothing (one row 7.3 against 7.5 us a step), nor with more than two
+// CTAs per SM (1000 x 32 positions 41.9 against 42.1).
+constexpr int kSpreadThreads = 512;
+constexpr int kSpreadCtas = 2 * 152;
+// The terms kernel's CTAs have 1024 threads: after 63 x 1000 confidences of 1004 logits their share of
+// a call 32.5 us with a row's own 256, 17.2 with 512, 10.9 with 1024; 64 x 256 8.2, 5.5 and 4.4.
+constexpr int kSpreadTerms = 1024;
+
+bool spread_rows(int64_t ctas) { return ctas > 4 && ctas <= kSpreadCtas; }
+
 template <int W, int K>
-__global__ void __launch_bounds__(32 * W) profile_select_kernel(const ProfileSelectArgs a,
-                                                                 int64_t bound, float tau_f)
+__global__ void __launch_bounds__(kSpreadThreads)
+    profile_select_kernel(const ProfileSelectArgs a, int64_t bound, float tau_f)
 {
+    static_assert(32 * W <= kSpreadThreads, "a row's warps");
+    if (threadIdx.x >= 32 * W)
+        return;
     constexpr int N = 32 * K * W;
     __shared__ uint64_t sk[W > 1 ? 2 * N : 1];
     __shared__ int32_t s_tok[N];
@@ -251,7 +278,7 @@ __global__ void __launch_bounds__(32 * W) profile_select_kernel(const ProfileSel
     if constexpr (W > 1) {
         if (lane == 0)
             warp_m[w] = any_bad ? -1 : m;
-        __syncthreads();
+        row_barrier<W>();
         m = 0;
         any_bad = false;
 #pragma unroll
@@ -284,7 +311,7 @@ __global__ void __launch_bounds__(32 * W) profile_select_kernel(const ProfileSel
     if constexpr (W > 1) {
         if (lane == 0)
             warp_n[w] = nstar;
-        __syncthreads();
+        row_barrier<W>();
 #pragma unroll
         for (int i = 0; i < W; ++i)
             nstar = max(nstar, warp_n[i]);
@@ -316,16 +343,26 @@ __global__ void __launch_bounds__(32 * W) profile_select_kernel(const ProfileSel
 
 // The same steps for rows of at most 32 positions, one warp per row: no block barriers, the
 // sort by rank counting (the keys are distinct: the position is in their low bits, pads
-// included), the scan by warp shuffles alone.
-__global__ void __launch_bounds__(32) profile_select_warp_kernel(const ProfileSelectArgs a,
-                                                                  int64_t bound, float tau_f)
+// included), the scan by warp shuffles alone.  More than two rows per SM go kWarpRows to a CTA: CTAs
+// of one row start at about one per ns (65536 rows of one position 101 -> 70 us a step, 2048 x 32
+// positions 51.1 -> 50.3, 305 x 32 19.4 -> 18.6).
+constexpr int kWarpRows = 8;
+
+__global__ void __launch_bounds__(kSpreadThreads)
+    profile_select_warp_kernel(const ProfileSelectArgs a, int rows_per_cta, int64_t bound,
+                               float tau_f)
 {
-    __shared__ uint64_t sk[32];
-    __shared__ int32_t s_tok[32];
+    __shared__ uint64_t s_keys[kWarpRows][32];
+    __shared__ int32_t s_toks[kWarpRows][32];
     constexpr unsigned kFull = 0xFFFFFFFFu;
-    const int t = threadIdx.x;
+    const int t = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t row = (int64_t)blockIdx.x * rows_per_cta + w;
+    if (w >= rows_per_cta || row >= a.B)
+        return;
+    uint64_t *const sk = s_keys[w];
+    int32_t *const s_tok = s_toks[w];
     const int L = a.L;
-    const int64_t base = (int64_t)blockIdx.x * L;
+    const int64_t base = row * L;
 
     // After the vocab reduction (partials given), the mask byte and the allowance are loaded
     // before the launch wait: this kernel starts only once the reduction has passed its own
@@ -354,8 +391,8 @@ __global__ void __launch_bounds__(32) profile_select_warp_kernel(const ProfileSe
     const bool masked = mask_byte != 0;
     float c = 0.0f;
     int32_t tok = -1;
-    if (in_row) {
-        if (a.partials != nullptr) {
+    if (in_row && (masked || !early)) {  // unmasked positions have no partials
+        if (early) {
             combine_position(a.partials + (base + t) * a.units_per_row, a.units_per_row, c,
                              tok);
         } else {
@@ -368,7 +405,7 @@ __global__ void __launch_bounds__(32) profile_select_warp_kernel(const ProfileSe
         tok = -1;
     }
     s_tok[t] = tok;
-    if (a.partials != nullptr && a.next_unit != nullptr && blockIdx.x == 0 && t == 0)
+    if (a.partials != nullptr && a.next_unit != nullptr && row == 0 && t == 0)
         *a.next_unit = 0;  // the vocab reduction before this kernel has finished
     const bool bad = masked && !(c > 0.0f && c <= 1.0f);  // NaN fails both
     float c_rank = c;
@@ -420,7 +457,7 @@ __global__ void __launch_bounds__(32) profile_select_warp_kernel(const ProfileSe
         }
     }
     if (t == 0)
-        a.out_n[blockIdx.x] = nstar;
+        a.out_n[row] = nstar;
 }
 
 // Heterogeneity-bonus diagnostics of one batch row per CTA (Prop. heterogeneity-bonus,
@@ -429,8 +466,10 @@ __global__ void __launch_bounds__(32) profile_select_warp_kernel(const ProfileSe
 // F_n = (n+1) c_(n) - n and B_n = S_n - n c_(n) (= sum_{j<n} (c_(j) - c_(n))); and the
 // effective factor f_eff(n) = 1 - delta + B_n of Remark adaptive-factor.
 template <int W, int K>
-__global__ void __launch_bounds__(32 * W) profile_terms_kernel(const ProfileTermsArgs a)
+__global__ void __launch_bounds__(kSpreadTerms) profile_terms_kernel(const ProfileTermsArgs a)
 {
+    if (threadIdx.x >= 32 * W)
+        return;
     constexpr int N = 32 * K * W;
     __shared__ uint64_t sk[W > 1 ? 2 * N : 1];
     __shared__ double warp_tot[W];
@@ -462,7 +501,7 @@ __global__ void __launch_bounds__(32 * W) profile_terms_kernel(const ProfileTerm
     if constexpr (W > 1) {
         if (lane == 0)
             warp_m[w] = m;
-        __syncthreads();
+        row_barrier<W>();
         m = 0;
 #pragma unroll
         for (int i = 0; i < W; ++i)
@@ -509,7 +548,7 @@ cudaError_t launch_terms_t(const ProfileTermsArgs &a, cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)a.B);
-    cfg.blockDim = dim3(32 * W);
+    cfg.blockDim = dim3(spread_rows(a.B) ? kSpreadTerms : 32 * W);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -519,12 +558,12 @@ cudaError_t launch_terms_t(const ProfileTermsArgs &a, cudaStream_t stream)
     return cudaLaunchKernelEx(&cfg, profile_terms_kernel<W, K>, a);
 }
 
-template <typename Kernel>
-cudaError_t launch_select(Kernel kern, int threads, const ProfileSelectArgs &a,
-                          int64_t bound, float tau_f, cudaStream_t stream)
+template <typename Kernel, typename... Args>
+cudaError_t launch_select(Kernel kern, int64_t ctas, int threads, const ProfileSelectArgs &a,
+                          cudaStream_t stream, Args... args)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)a.B);
+    cfg.gridDim = dim3((unsigned)ctas);
     cfg.blockDim = dim3(threads);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -532,7 +571,16 @@ cudaError_t launch_select(Kernel kern, int threads, const ProfileSelectArgs &a,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = a.pdl ? 1 : 0;  // a programmatic dependent of the previous kernel
-    return cudaLaunchKernelEx(&cfg, kern, a, bound, tau_f);
+    return cudaLaunchKernelEx(&cfg, kern, a, args...);
+}
+
+// One CTA per row of W warps.
+template <int W, int K>
+cudaError_t launch_rows(const ProfileSelectArgs &a, bool spread, int64_t bound, float tau_f,
+                        cudaStream_t stream)
+{
+    return launch_select(profile_select_kernel<W, K>, a.B, spread ? kSpreadThreads : 32 * W, a,
+                         stream, bound, tau_f);
 }
 
 }  // namespace
@@ -549,17 +597,22 @@ cudaError_t launch_profile_select(const ProfileSelectArgs &a, cudaStream_t strea
     float tau_f = (float)a.param;  // the smallest fp32 value >= tau
     if ((double)tau_f < a.param)
         tau_f = std::nextafter(tau_f, INFINITY);
+    const int per = a.L <= 32 && a.B > kSpreadCtas ? kWarpRows : 1;
+    const int64_t ctas = (a.B + per - 1) / per;
+    const bool room = a.partials != nullptr && !a.warp_units;  // after CTA units
+    const bool spread = !room && spread_rows(ctas);
     if (a.L <= 32)
-        return launch_select(profile_select_warp_kernel, 32, a, bound, tau_f, stream);
+        return launch_select(profile_select_warp_kernel, ctas, spread ? kSpreadThreads : 32 * per,
+                             a, stream, per, bound, tau_f);
     if (a.L <= 64)
-        return launch_select(profile_select_kernel<1, 2>, 32, a, bound, tau_f, stream);
+        return launch_rows<1, 2>(a, spread, bound, tau_f, stream);
     if (a.L <= 128)
-        return launch_select(profile_select_kernel<2, 2>, 64, a, bound, tau_f, stream);
+        return launch_rows<2, 2>(a, spread, bound, tau_f, stream);
     if (a.L <= 256)
-        return launch_select(profile_select_kernel<4, 2>, 128, a, bound, tau_f, stream);
+        return launch_rows<4, 2>(a, spread, bound, tau_f, stream);
     if (a.L <= 512)
-        return launch_select(profile_select_kernel<8, 2>, 256, a, bound, tau_f, stream);
-    return launch_select(profile_select_kernel<16, 2>, 512, a, bound, tau_f, stream);
+        return launch_rows<8, 2>(a, spread, bound, tau_f, stream);
+    return launch_rows<16, 2>(a, spread, bound, tau_f, stream);
 }
 
 cudaError_t launch_profile_terms(const ProfileTermsArgs &a, cudaStream_t stream)

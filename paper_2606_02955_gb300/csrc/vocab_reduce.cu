@@ -944,24 +944,23 @@ __global__ void __launch_bounds__(kUnitWarps * 32, 1)
     }
 }
 
-__global__ void finalize_kernel(const FinalizeArgs a)
+__global__ void __launch_bounds__(512) finalize_kernel(const FinalizeArgs a, int rows_per_cta)
 {
+    const int64_t row = (int64_t)blockIdx.x * rows_per_cta + threadIdx.x;
+    const bool in_rows = (int)threadIdx.x < rows_per_cta && row < a.rows;
+    // Loaded before the wait: this kernel starts only once the reduction has passed its own, so the
+    // mask's writer has completed, and the reduction does not write it.
+    const bool masked = in_rows && __ldcg(a.mask + row) != 0;
     pdl_wait();  // the vocab reduction's partials are complete and visible
     if (threadIdx.x == 0)
         pdl_launch_dependents();  // a following vocab reduction may start its prologue
     if (blockIdx.x == 0 && threadIdx.x == 0)
         *a.next_unit = 0;
-    const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= a.rows)
+    if (!masked)
         return;
-    // The mask byte and the partials are loaded together; an unmasked row's partials are
-    // in-bounds leftovers and are discarded.
-    const bool masked = a.mask[row] != 0;
     float c;
     int32_t tok;
     combine_position(a.partials + row * a.units_per_row, a.units_per_row, c, tok);
-    if (!masked)
-        return;
     a.out_conf[row] = c;
     a.out_tok[row] = tok;
 }
@@ -1096,9 +1095,15 @@ cudaError_t launch_vocab_reduce(const VocabReduceArgs &a, int dtype, cudaStream_
 
 cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t stream)
 {
-    const int threads = 256;
+    // After warp units, CTAs of 512 threads that take rows / 304 rows each, so that they do not all
+    // start on the first SMs to be freed (see kSpreadThreads in profile_select.cu): 2048 rows of
+    // 32000 bf16 logits 27.4 -> 22.3 us a call, of 20000 19.0 -> 16.9, 7991 of 20008 fp16 46.0 ->
+    // 44.0, 63000 of 1004 fp32 36.2 -> 35.7.
+    const int64_t share = (a.rows + 2 * 152 - 1) / (2 * 152);
+    const int threads = a.warp_units ? 512 : 256;
+    const int rows_per_cta = a.warp_units ? (int)((share + 31) / 32 * 32) : threads;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((a.rows + threads - 1) / threads));
+    cfg.gridDim = dim3((unsigned)((a.rows + rows_per_cta - 1) / rows_per_cta));
     cfg.blockDim = dim3(threads);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -1106,7 +1111,7 @@ cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t stream)
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, finalize_kernel, a);
+    return cudaLaunchKernelEx(&cfg, finalize_kernel, a, rows_per_cta);
 }
 
 }  // namespace fdllm

@@ -45,6 +45,29 @@ def test_row_lengths_against_the_oracle(fd, orc, dtype, vecs):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("B, L", [(304, 32), (304, 33), (305, 1), (305, 32), (305, 70), (311, 3),
+                                  (2432, 4), (2433, 4), (9729, 1)])
+def test_many_rows(fd, orc, B, L):
+    """The edges of how the kernels after the reduction spread rows over CTAs: up to 304 batch rows
+    one to a CTA, then (L <= 32) eight, up to and beyond 304 such CTAs; 32 or (beyond 9728
+    positions) more of them to a CTA."""
+    w = syn.Workload("many", B, L, 1000, "bf16", 1.0, "target", 0.3, 3.0)
+    x = syn.make_logits(w, seed=B + L, device="cuda")
+    mask = (np.random.default_rng(B).random((B, L)) < 0.7).astype(np.uint8)
+    mask[-1] = 1
+    x[B // 2, 0, 999] = torch.nan
+    mask[B // 2, 0] = 1
+    check_confidence(fd, orc, x, mask)
+    assert check_select(fd, orc, x, mask, oracle.PROFILE, 0.75) <= B // 50 + 1
+    x[B // 2, 0, 999] = 1.0
+    conf, tok = fd.fdllm_confidence(x, torch.from_numpy(mask).cuda())
+    a, b = torch.from_numpy(mask.copy()).cuda(), torch.from_numpy(mask.copy()).cuda()
+    got = fd.fdllm_select(x, a, 0.75, oracle.FACTOR)
+    ref = fd.fdllm_select_from_conf(conf.nan_to_num(0.5), tok, b, 0.75, oracle.FACTOR)
+    assert torch.equal(a, b) and all(torch.equal(g, r) for g, r in zip(got, ref))
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("dtype", ["bf16", "fp16", "fp32"])
 def test_unusable_rows(fd, orc, dtype):
     """NaN, +inf and all -inf anywhere in a row's units make it unusable, its neighbours not."""
