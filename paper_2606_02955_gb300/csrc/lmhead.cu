@@ -746,9 +746,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // ----------------------------------------------------------------------------- wide variant
 // W is the M = 256 operand of a CTA pair (a tile of 2 h vocabulary entries, h <= 128 per CTA, lane
-// = entry, see wide_height) and the packed rows are N, in blocks of up to 256 rows (one MMA group, two accumulators
-// in turn) or, for 257 to 320 rows, one block of two groups that share every W stage (three
-// accumulators).  What bounds the solo variant at 2 to 6 row tiles is the 64 B/clock at which an
+// = entry, see wide_height) and the packed rows are N, in blocks of up to 256 rows (one MMA group,
+// two accumulators in turn) or, for 257 to 320 rows, one block of two groups that share every W
+// stage (three accumulators).  What bounds the solo variant at 2 to 6 row tiles is the 64 B/clock at which an
 // SM receives from L2: its stage is 42 KB for 416 MMA cycles (101 B/clock wanted, 65 measured).
 // Here a stage is (128 + N / 2) x 128 B for 2 N cycles: 75 B/clock at N = 192, 58 at 320, and no
 // row tile is padded to 128.  LLaDA's head, 3/4 of B x 32 rows, whole fdllm_lmhead_confidence
@@ -783,7 +783,6 @@ struct WideRowMaps {
 // columns take turns.
 struct WideCut {
     int n_blocks, groups, g, g1, buffers;
-    __device__ __forceinline__ int width(int j) const { return j == 0 ? g : g1; }
 };
 
 __device__ __forceinline__ WideCut wide_cut(int R)
@@ -798,37 +797,62 @@ __device__ __forceinline__ WideCut wide_cut(int R)
     return c;
 }
 
-// The items of one CTA pair.  Whole rounds of items over the pairs first; if what is left then
-// fills at most half of them and a block has two groups, each leftover item goes to two pairs,
-// one group each.
+// What a CTA pair works on at a time: the rows of W tile n from row0 on, in one group of w0 or two of
+// w0 and w1 columns.
+struct WidePiece {
+    int n, row0, w0, w1;
+};
+
+// The pieces of one CTA pair.  Whole rounds of items over the pairs first; if what is left then
+// fills at most half of them, each leftover item goes to two pairs, one group or half of the one
+// group each.  Halves of fewer than 80 columns would gain nothing, since a stage's W share alone
+// takes as long to arrive as 128 columns' MMAs.  Whole fdllm_lmhead_confidence pass with one-group
+// items left whole against halved: 200 rows, H = 4096, 20000 entries 49.5 -> 46.4 us, 65000 entries
+// 98.7 -> 95.8, LLaDA's 169 -> 167; H = 1024, 20000 entries 200 rows 20.6 -> 19.5, 700 rows 32.9 ->
+// 31.4; H = 2048, 8000 entries 200 rows 19.5 -> 17.5.
+constexpr int kWideHalved = 160;
+
 struct WideItems {
+    const WideCut cut;
     // items of whole rounds, all items (B * L * V / 208 < 2^31 keeps them small), this pair
     int whole, total, pairs, pair;
-    bool split;
+    int first;  // columns of a leftover item's first part; 0: not cut
 
     __device__ __forceinline__ WideItems(const WideCut &c, int n_w_tiles, int pairs_, int pair_)
-        : total(n_w_tiles * c.n_blocks), pairs(pairs_), pair(pair_)
+        : cut(c), total(n_w_tiles * c.n_blocks), pairs(pairs_), pair(pair_)
     {
         const int left = total % pairs;
         whole = total - left;
-        split = c.groups == 2 && 2 * left <= pairs;
+        first = 2 * left > pairs       ? 0
+                : c.groups == 2        ? c.g
+                : c.g >= kWideHalved   ? (c.g / 2 + 31) / 32 * 32
+                                       : 0;
     }
-    // The pair's i-th item: its index, or -1 past the last, and its groups [j0, j1).
-    __device__ __forceinline__ int item(int i, int groups, int &j0, int &j1) const
+    // The pair's i-th piece; false past the last.
+    __device__ __forceinline__ bool piece(int i, WidePiece &p) const
     {
-        j0 = 0;
-        j1 = groups;
-        const int t = i * pairs + pair;
-        if (t < whole)
-            return t;
-        if (i != whole / pairs)
-            return -1;
-        if (!split)
-            return t < total ? t : -1;
-        const int u = whole + pair / 2;
-        j0 = pair & 1;
-        j1 = j0 + 1;
-        return u < total ? u : -1;
+        int t = i * pairs + pair;
+        p.w0 = cut.g;
+        p.w1 = cut.g1;
+        int off = 0;
+        if (t >= whole) {
+            if (i != whole / pairs)
+                return false;
+            if (first != 0) {
+                t = whole + pair / 2;
+                p.w0 = first;
+                p.w1 = 0;
+                if (pair & 1) {
+                    off = first;
+                    p.w0 = cut.g + cut.g1 - first;
+                }
+            }
+            if (t >= total)
+                return false;
+        }
+        p.n = t / cut.n_blocks;
+        p.row0 = t % cut.n_blocks * cut.g + off;  // one block where there are two groups
+        return true;
     }
 };
 
@@ -966,7 +990,6 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     const int rank = (int)tc::cluster_ctarank();
     const int R = __shfl_sync(0xFFFFFFFFu, *a.row_count, 0);
     const WideCut cut = wide_cut(R);
-    const int block_rows = cut.g;  // one block where there are two groups
     const int h = a.wide_h;
     // a CTA's share of a group of g rows in a stage
     auto half_bytes = [](int g) { return (uint32_t)(g / 2 * BK * 2); };
@@ -982,20 +1005,15 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         int s = 0;
         uint32_t ph = 0, filled = 0;
         bool ok = true;
-        int j0, j1;
-        for (int i = 0; ok; ++i) {
-            const int t = items.item(i, cut.groups, j0, j1);
-            if (t < 0)
-                break;
-            const int n = t / cut.n_blocks;
-            const int g = cut.width(j0);
-            const int row0 = t % cut.n_blocks * block_rows + j0 * cut.g + rank * (g / 2);
-            const int row1 = cut.g + rank * (cut.g1 / 2);  // the second of two groups
-            const CUtensorMap *map0 = &maps_h.m[g / 32 - 1];
-            const CUtensorMap *map1 = &maps_h.m[j1 - j0 == 2 ? cut.g1 / 32 - 1 : 0];
-            const int w_row = (2 * n + rank) * h;
-            const uint32_t bytes =
-                a_bytes + half_bytes(g) + (j1 - j0 == 2 ? half_bytes(cut.g1) : 0u);
+        WidePiece p;
+        for (int i = 0; ok && items.piece(i, p); ++i) {
+            const bool two = p.w1 != 0;
+            const int row0 = p.row0 + rank * (p.w0 / 2);
+            const int row1 = p.row0 + p.w0 + rank * (p.w1 / 2);
+            const CUtensorMap *map0 = &maps_h.m[p.w0 / 32 - 1];
+            const CUtensorMap *map1 = &maps_h.m[two ? p.w1 / 32 - 1 : 0];
+            const int w_row = (2 * p.n + rank) * h;
+            const uint32_t bytes = a_bytes + half_bytes(p.w0) + half_bytes(p.w1);
             for (int kb = 0; kb < a.k_blocks; ++kb) {
                 if (!warp_wait(&empty[s], ph ^ 1u, a.status, abort_flag)) {
                     ok = false;
@@ -1009,9 +1027,9 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                     uint8_t *stage = smem + s * stage_bytes;
                     tc::tma_load_2d_pair_hint(stage, &map_w, kb * BK, w_row, bar0, pol);
                     tc::tma_load_2d_pair(stage + a_bytes, map0, kb * BK, row0, bar0);
-                    if (j1 - j0 == 2)
-                        tc::tma_load_2d_pair(stage + a_bytes + half_bytes(g), map1, kb * BK, row1,
-                                             bar0);
+                    if (two)
+                        tc::tma_load_2d_pair(stage + a_bytes + half_bytes(p.w0), map1, kb * BK,
+                                             row1, bar0);
                 }
                 filled = min(filled + 1, (uint32_t)stages);
                 if (++s == stages) {
@@ -1031,20 +1049,17 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             uint32_t ph = 0;
             uint32_t used = 0;  // groups accumulated so far
             bool ok = true;
-            int j0, j1;
-            for (int i = 0; ok; ++i) {
-                const int t = items.item(i, cut.groups, j0, j1);
-                if (t < 0)
-                    break;
-                const bool two = j1 - j0 == 2;
+            WidePiece p;
+            for (int i = 0; ok && items.piece(i, p); ++i) {
+                const bool two = p.w1 != 0;
                 const uint32_t b0 = used % cut.buffers, b1 = (used + 1) % cut.buffers;
                 const uint32_t turn1 = (used + 1) / cut.buffers;
                 if (!warp_wait(&tempty[b0], (used / cut.buffers & 1u) ^ 1u, a.status, abort_flag))
                     break;
                 tc::fence_after_sync();
                 const uint32_t d0 = tmem_base + b0 * cut.g, d1 = tmem_base + b1 * cut.g;
-                const uint32_t idesc0 = tc::idesc_bf16_f32(2 * BM, cut.width(j0));
-                const uint32_t idesc1 = tc::idesc_bf16_f32(2 * BM, cut.g1);
+                const uint32_t idesc0 = tc::idesc_bf16_f32(2 * BM, p.w0);
+                const uint32_t idesc1 = tc::idesc_bf16_f32(2 * BM, p.w1);
                 // Two groups share each stage.  While the second group's accumulator is still
                 // being read, the first one runs ahead over the stages of the ring (k0, at s);
                 // the second one follows (k1, at s1), the last to read a stage.
@@ -1093,7 +1108,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                         }
                     }
                     const uint64_t ad = tc::sw128_kmajor_desc(smem + s1 * stage_bytes);
-                    const uint64_t bd = ad + (a_bytes >> 4) + (half_bytes(cut.g) >> 4);
+                    const uint64_t bd = ad + (a_bytes >> 4) + (half_bytes(p.w0) >> 4);
                     if (elect_one()) {
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k)
@@ -1108,8 +1123,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                     break;
                 if (two && elect_one())
                     tc::commit_pair_multicast(&tfull[b1]);
-                const int ng = j1 - j0;
-                used += ng;
+                used += two ? 2 : 1;
             }
             // Tensor memory is freed below only after every MMA issued here has completed.
             __syncwarp();
@@ -1125,17 +1139,13 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         const int quarter = warp & 3, third = (warp - 2) >> 2;
         const int et = threadIdx.x - 64;
         uint32_t used = 0;
-        int j0, j1;
         bool ok = true;
-        for (int i = 0; ok; ++i) {
-            const int t = items.item(i, cut.groups, j0, j1);
-            if (t < 0)
-                break;
-            const int n = t / cut.n_blocks;
-            const int blk0 = t % cut.n_blocks * block_rows;
+        WidePiece p;
+        for (int i = 0; ok && items.piece(i, p); ++i) {
+            const int n = p.n, ng = p.w1 != 0 ? 2 : 1;
             const int ent0 = (2 * n + rank) * h;  // this CTA's entries: ent0 .. ends - 1
             const int ends = min(a.V, ent0 + h);
-            for (int j = j0; j < j1; ++j, ++used) {
+            for (int j = 0; j < ng; ++j, ++used) {
                 const uint32_t buf = used % cut.buffers, turn = used / cut.buffers;
                 const bool got = wait_or_abort(&tfull[buf], turn & 1u, a.status, abort_flag);
                 // All epilogue warps go on or leave together (they share barriers below); past
@@ -1147,8 +1157,8 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                 tc::fence_after_sync();
                 const uint32_t taddr =
                     tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * cut.g;
-                const int row0 = blk0 + j * cut.g;
-                const int live = min(cut.width(j), R - row0);  // columns that are rows
+                const int row0 = p.row0 + j * p.w0;
+                const int live = min(j == 0 ? p.w0 : p.w1, R - row0);  // columns that are rows
 #pragma unroll 1
                 for (int c = third * 32; c < live; c += kWideSplit * 32) {
                     float x[2][16];
@@ -1201,12 +1211,12 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                                        q_S[q * kWideMaxGroup + et],
                                        e < 32 ? (uint32_t)(ent0 + q * 32) + e : kNoIdx);
                         }
-                        UnitPartial p;
-                        p.M = S != S ? __int_as_float(0x7FC00000) : M;
-                        p.S = M == -INFINITY ? 0.0f : S;
-                        p.idx = I;
-                        p.pad = 0;
-                        a.partials[(int64_t)(row0 + et) * a.n_tiles + 2 * n + rank] = p;
+                        UnitPartial u;
+                        u.M = S != S ? __int_as_float(0x7FC00000) : M;
+                        u.S = M == -INFINITY ? 0.0f : S;
+                        u.idx = I;
+                        u.pad = 0;
+                        a.partials[(int64_t)(row0 + et) * a.n_tiles + 2 * n + rank] = u;
                     }
                 }
             }

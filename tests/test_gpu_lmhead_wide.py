@@ -31,6 +31,12 @@ SHAPES = [
     (14, 64, 64, 3000, 896),     # the most rows that take this variant by default
     (16, 66, 64, 3000, 1040),    # more
     (5, 64, 8, 20000, 320),      # H below one K-block
+    (4, 64, 128, 19500, 225),    # 77 tiles: one left over, its group of 256 halved
+    (4, 64, 64, 25000, 150),     # a group of 160 cut into 96 and 64
+    (6, 64, 64, 19600, 384),     # two blocks of 192, one tile's two items left over
+    (10, 64, 64, 6000, 600),     # three blocks of 224: too many items left over to halve
+    (10, 64, 64, 3000, 577),     # halved; the last half has one row
+    (13, 64, 64, 2000, 770),     # four blocks; the last half has none
 ]
 
 
