@@ -760,7 +760,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 // 245, 480 rows in one block 311 against 293 in two.
 constexpr int kWideMaxGroup = 256;              // MMA columns per group
 constexpr int kWideTwoGroups = 320;             // rows that still make one block, of two groups
-constexpr int kWideMaxStages = 12;
+// A few rows leave room for 12 and more stages, but W streams faster with fewer of its bytes in
+// flight: of 4 x 32 rows 8 masked 161 us with 14 stages, 155.5 with 12, 154.2 with 11, 154.4 with 10,
+// 157 with 8; 64 masked 159.5, 156.6, 157.2 and 160 (12, 11, 10, 8), 96 masked 157.8, 157.9, 158.3
+// and 161.3; H = 1024, 100000 entries, 8 masked 39.7, 39.1, 38.5 and 38.4.
+constexpr int kWideMaxStages = 11;
 constexpr int kWideWarps = 12;                  // epilogue warps, three per TMEM lane quarter
 constexpr int kWideSplit = kWideWarps / 4;
 constexpr int kWideThreads = 64 + kWideWarps * 32;
