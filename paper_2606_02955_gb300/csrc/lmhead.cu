@@ -475,8 +475,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 // 16 KB.  A stage holds two K-blocks (two W boxes and two row boxes), five stages in all
 // (130 KB of W at h = 104 in flight per SM): per-copy overhead, not the bytes in flight,
 // limits how fast W streams here, and two blocks per stage beat one, three or four.  Each
-// epilogue thread keeps, for every row, a running maximum, sum of exp relative to it and
-// first index over its own entry of each tile; after the last tile the 128 threads' states
+// epilogue thread keeps, for each of its 16 rows, a running maximum, sum of exp relative to it and
+// first index over its own entry of each tile; after the last tile the 128 entries' states
 // are folded per row (a transposing butterfly in each warp, then the four warps in order)
 // into one partial per (row, CTA).
 constexpr int kSlabRows = 32;
@@ -486,6 +486,13 @@ constexpr int kSlabKB = 2;                               // K-blocks of BK per s
 constexpr int kSlabStages = 5;
 constexpr int kSlabAccs = 4;                             // accumulators of 32 columns
 constexpr uint32_t kSlabTmemCols = 128;
+// Two epilogue warps per TMEM lane quarter, 16 rows each: the last tile's reduction and the fold
+// over the entries are the kernel's tail.  Whole fdllm_lmhead_confidence pass, one warp of 32 rows
+// against two of 16: 24 rows, H = 1024, 20000 entries 13.9 -> 12.9 us, 8000 10.6 -> 10.2, H = 2048,
+// 65000 46.2 -> 45.4, LLaDA's head 151.9 -> 151.2.
+constexpr int kSlabWarps = 8;
+constexpr int kSlabWarpRows = kSlabRows / (kSlabWarps / 4);
+constexpr int kSlabThreads = 64 + kSlabWarps * 32;
 constexpr size_t kSlabSmemBytes =
     1024 + (size_t)kSlabStages * kSlabKB * (kSlabABytes + kSlabBBytes) + kBarrierBytes;
 static_assert(kSlabSmemBytes <= 227 * 1024, "slab ring");
@@ -504,7 +511,7 @@ __device__ __forceinline__ void fold_state(float &M, float &S, uint32_t &I, floa
 }
 
 template <int EPI>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kSlabThreads, 1)
     lmhead_slab_kernel(const __grid_constant__ CUtensorMap map_h,
                        const __grid_constant__ CUtensorMap map_w, const GemmArgs a)
 {
@@ -533,7 +540,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         for (int i = 0; i < kSlabAccs; ++i) {
             mbar_init(&tfull[i], 1);
-            mbar_init(&tempty[i], 4);
+            mbar_init(&tempty[i], kSlabWarps);
         }
         mbar_init(done, 1);
         *abort_flag = 0;
@@ -641,12 +648,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
     } else {
         // Epilogue: warp w reads TMEM lanes [32 (w % 4), +32): thread = one vocabulary entry
-        // of the tile, its 32 columns = the rows.
-        const int q = warp & 3;
-        float M[kSlabRows], S[kSlabRows];
-        uint32_t I[kSlabRows];
+        // of the tile, its columns = kSlabWarpRows of the rows, from row0 on.
+        const int q = warp & 3, row0 = (warp - 2) / 4 * kSlabWarpRows;
+        float M[kSlabWarpRows], S[kSlabWarpRows];
+        uint32_t I[kSlabWarpRows];
 #pragma unroll
-        for (int r = 0; r < kSlabRows; ++r) {
+        for (int r = 0; r < kSlabWarpRows; ++r) {
             M[r] = -__int_as_float(0x7F800000);
             S[r] = 0.0f;
             I[r] = kNoIdx;
@@ -661,10 +668,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 break;
             }
             tc::fence_after_sync();
-            float v[32];
-            tc::tmem_ld_32cols(tmem_base + ((uint32_t)(q * 32) << 16) +
-                                   (uint32_t)(acc * kSlabRows),
-                               v);
+            float v[kSlabWarpRows];
+            tc::tmem_ld_16cols_async(tmem_base + ((uint32_t)(q * 32) << 16) +
+                                         (uint32_t)(acc * kSlabRows + row0),
+                                     v);
+            tc::tmem_wait_ld();
+            tc::tie_regs(v);
             tc::fence_before_sync();
             __syncwarp();
             if (lane == 0)
@@ -676,12 +685,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 continue;
             if (EPI == kStore) {
 #pragma unroll
-                for (int r = 0; r < kSlabRows; ++r)
-                    if (r < R)
-                        a.logits[(int64_t)a.row_ids[r] * a.V + ent] = v[r];
+                for (int r = 0; r < kSlabWarpRows; ++r)
+                    if (row0 + r < R)
+                        a.logits[(int64_t)a.row_ids[row0 + r] * a.V + ent] = v[r];
             } else {
 #pragma unroll
-                for (int r = 0; r < kSlabRows; ++r) {
+                for (int r = 0; r < kSlabWarpRows; ++r) {
                     // exp(x - M) in the form (x - M) * log2e, exact at any magnitude; a
                     // larger x re-bases the sum; -inf adds nothing; NaN poisons S
                     const float x = v[r];
@@ -696,9 +705,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (EPI == kReduce) {
             // Transposing butterfly: at offset o each lane keeps the half of its remaining
             // row slots selected by its lane bit o and folds in the partner's values for them;
-            // slot 0 ends as row `lane`, folded over the warp's 32 entries.
+            // slot 0 ends as row row0 + lane % 16, folded over half of the warp's 32 entries, then
+            // over both.
+            const int mine = lane & (kSlabWarpRows - 1);
 #pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) {
+            for (int o = kSlabWarpRows / 2; o >= 1; o >>= 1) {
                 const bool hi = (lane & o) != 0;
 #pragma unroll
                 for (int j = 0; j < o; ++j) {
@@ -715,12 +726,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                     I[j] = kI;
                 }
             }
-            s_M[q][lane] = M[0];
-            s_S[q][lane] = S[0];
-            s_I[q][lane] = I[0];
+            fold_state(M[0], S[0], I[0], __shfl_xor_sync(0xFFFFFFFFu, M[0], kSlabWarpRows),
+                       __shfl_xor_sync(0xFFFFFFFFu, S[0], kSlabWarpRows),
+                       __shfl_xor_sync(0xFFFFFFFFu, I[0], kSlabWarpRows));
+            if (lane < kSlabWarpRows) {
+                s_M[q][row0 + mine] = M[0];
+                s_S[q][row0 + mine] = S[0];
+                s_I[q][row0 + mine] = I[0];
+            }
             // every epilogue warp arrives exactly once, aborted or not
-            asm volatile("bar.sync 1, 128;" ::: "memory");
-            if (q == 0 && !aborted && !*abort_flag && lane < R) {
+            asm volatile("bar.sync 1, %0;" ::"n"(kSlabWarps * 32) : "memory");
+            if (warp == 4 && !aborted && !*abort_flag && lane < R) {
                 float fM = s_M[0][lane], fS = s_S[0][lane];
                 uint32_t fI = s_I[0][lane];
                 for (int w = 1; w < 4; ++w)
@@ -1775,7 +1791,7 @@ cudaError_t launch_slab(const CUtensorMap &mh, const CUtensorMap &mw, const Gemm
     });
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)g.n_tiles);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kSlabThreads);
     cfg.dynamicSmemBytes = kSlabSmemBytes;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
