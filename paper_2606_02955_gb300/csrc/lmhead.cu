@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
 
     pdl_wait();  // the packed rows and their count are complete
 
-    const int R = __shfl_sync(0xFFFFFFFFu, *a.row_count, 0);  // <= kSlabRows: the host takes this variant only then
+    const int R = __shfl_sync(0xFFFFFFFFu, *a.row_count, 0);  // <= kSlabRows: the host's choice
     const int64_t NT = a.slab_tiles, P = gridDim.x, c = blockIdx.x;
     const int h = a.slab_h;
     const int n_t = R > 0 && c < NT ? (int)((NT - c + P - 1) / P) : 0;  // tiles of this CTA
@@ -764,8 +764,8 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
 // W is the M = 256 operand of a CTA pair (a tile of 2 h vocabulary entries, h <= 128 per CTA, lane
 // = entry, see wide_height) and the packed rows are N, in blocks of up to 256 rows (one MMA group,
 // two accumulators in turn) or, for 257 to 320 rows, one block of two groups that share every W
-// stage (three accumulators).  What bounds the solo variant at 2 to 6 row tiles is the 64 B/clock at which an
-// SM receives from L2: its stage is 42 KB for 416 MMA cycles (101 B/clock wanted, 65 measured).
+// stage (three accumulators).
+// What bounds the solo variant at 2 to 6 row tiles is the 64 B/clock at which an SM receives from L2: its stage is 42 KB for 416 MMA cycles (101 B/clock wanted, 65 measured).
 // Here a stage is (128 + N / 2) x 128 B for 2 N cycles: 75 B/clock at N = 192, 58 at 320, and no
 // row tile is padded to 128.  LLaDA's head, 3/4 of B x 32 rows, whole fdllm_lmhead_confidence
 // pass, this variant against the better of solo and pair: B = 3 (72 rows) 160 against 163 us,
@@ -777,9 +777,9 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
 constexpr int kWideMaxGroup = 256;              // MMA columns per group
 constexpr int kWideTwoGroups = 320;             // rows that still make one block, of two groups
 // A few rows leave room for 12 and more stages, but W streams faster with fewer of its bytes in
-// flight: of 4 x 32 rows 8 masked 161 us with 14 stages, 155.5 with 12, 154.2 with 11, 154.4 with 10,
-// 157 with 8; 64 masked 159.5, 156.6, 157.2 and 160 (12, 11, 10, 8), 96 masked 157.8, 157.9, 158.3
-// and 161.3; H = 1024, 100000 entries, 8 masked 39.7, 39.1, 38.5 and 38.4.
+// flight: of 4 x 32 rows 8 masked 161 us with 14 stages, 155.5 with 12, 154.2 with 11, 154.4 with
+// 10, 157 with 8; 64 masked 159.5, 156.6, 157.2 and 160 (12, 11, 10, 8), 96 masked 157.8, 157.9,
+// 158.3 and 161.3; H = 1024, 100000 entries, 8 masked 39.7, 39.1, 38.5 and 38.4.
 constexpr int kWideMaxStages = 11;
 constexpr int kWideWarps = 12;                  // epilogue warps, three per TMEM lane quarter
 constexpr int kWideSplit = kWideWarps / 4;
@@ -817,8 +817,8 @@ __device__ __forceinline__ WideCut wide_cut(int R)
     return c;
 }
 
-// What a CTA pair works on at a time: the rows of W tile n from row0 on, in one group of w0 or two of
-// w0 and w1 columns.
+// What a CTA pair works on at a time: W tile n and the rows from row0 on, in one group of w0 or two
+// of w0 and w1 columns.
 struct WidePiece {
     int n, row0, w0, w1;
 };

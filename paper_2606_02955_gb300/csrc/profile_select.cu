@@ -171,8 +171,8 @@ __device__ __forceinline__ bool rule_accepts(int mode, int n, float cn, int64_t 
     return cn >= tau_f;  // threshold: c_(n) >= tau
 }
 
-// Where rows' CTAs start while the kernel before them holds the SMs (the warp units all registers of
-// every SM, the confidences' own pass many of its threads), small ones are all placed on the first
+// Where rows' CTAs start while the kernel before them holds the SMs (the warp units all registers
+// of every SM, the confidences' own pass many of its threads), small ones are all placed on the first
 // few SMs to be freed, where their loads and sorts then queue.  CTAs of 512 threads, the warps
 // beyond a row's own returning at once, spread over more.  Time over the reduction alone, a row's
 // own warps against 512 threads: 64 x 32 positions of 32000 bf16 logits 7.8 -> 3.1 us, of 20000 5.0
@@ -182,8 +182,8 @@ __device__ __forceinline__ bool rule_accepts(int mode, int n, float cn, int64_t 
 // CTAs per SM (1000 x 32 positions 41.9 against 42.1).
 constexpr int kSpreadThreads = 512;
 constexpr int kSpreadCtas = 2 * 152;
-// The terms kernel's CTAs have 1024 threads: after 63 x 1000 confidences of 1004 logits their share of
-// a call 32.5 us with a row's own 256, 17.2 with 512, 10.9 with 1024; 64 x 256 8.2, 5.5 and 4.4.
+// The terms kernel's CTAs have 1024 threads: after 63 x 1000 confidences of 1004 logits their share
+// of a call 32.5 us with a row's own 256, 17.2 with 512, 10.9 with 1024; 64 x 256 8.2, 5.5 and 4.4.
 constexpr int kSpreadTerms = 1024;
 
 bool spread_rows(int64_t ctas) { return ctas > 4 && ctas <= kSpreadCtas; }
@@ -343,8 +343,8 @@ __global__ void __launch_bounds__(kSpreadThreads)
 
 // The same steps for rows of at most 32 positions, one warp per row: no block barriers, the
 // sort by rank counting (the keys are distinct: the position is in their low bits, pads
-// included), the scan by warp shuffles alone.  More than two rows per SM go kWarpRows to a CTA: CTAs
-// of one row start at about one per ns (65536 rows of one position 101 -> 70 us a step, 2048 x 32
+// included), the scan by warp shuffles alone.  More than two rows per SM go kWarpRows to a CTA:
+// CTAs of one row start at about one per ns (65536 rows of one position 101 -> 70 us a step, 2048 x 32
 // positions 51.1 -> 50.3, 305 x 32 19.4 -> 18.6).
 constexpr int kWarpRows = 8;
 
