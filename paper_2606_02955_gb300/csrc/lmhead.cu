@@ -765,7 +765,8 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
 // = entry, see wide_height) and the packed rows are N, in blocks of up to 256 rows (one MMA group,
 // two accumulators in turn) or, for 257 to 320 rows, one block of two groups that share every W
 // stage (three accumulators).
-// What bounds the solo variant at 2 to 6 row tiles is the 64 B/clock at which an SM receives from L2: its stage is 42 KB for 416 MMA cycles (101 B/clock wanted, 65 measured).
+// What bounds the solo variant at 2 to 6 row tiles is the 64 B/clock at which an SM receives from
+// L2: its stage is 42 KB for 416 MMA cycles (101 B/clock wanted, 65 measured).
 // Here a stage is (128 + N / 2) x 128 B for 2 N cycles: 75 B/clock at N = 192, 58 at 320, and no
 // row tile is padded to 128.  LLaDA's head, 3/4 of B x 32 rows, whole fdllm_lmhead_confidence
 // pass, this variant against the better of solo and pair: B = 3 (72 rows) 160 against 163 us,
