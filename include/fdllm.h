@@ -256,11 +256,11 @@ fdllm_status fdllm_select_host(const void *logits, int dtype, int B, int L, int 
  *            16-byte aligned.
  *   H        hidden size, a multiple of 8 (16-byte rows); V >= 1, any value.
  * mask, param, mode and the outputs as in fdllm_select (B*L <= FDLLM_MAX_ROWS, L <=
- * FDLLM_MAX_L).  Uses the library-owned workspace (at most B*L*(2H + 32*ceil(V/256) + 12)
+ * FDLLM_MAX_L).  Uses the library-owned workspace (at most B*L*(2H + 32*ceil(V/192) + 12)
  * bytes and a header), allocated outside the step as for fdllm_select.  Asynchronous on
  * `stream`.  The GEMM's tiling (vocabulary slabs for at most 32 rows, the vocabulary as the
- * wide operand of CTA pairs up to 896, CTA pairs on row tiles of 128 beyond) is chosen from
- * B*L and V, and under stream capture from what the workspace holds; the environment variables
+ * wide operand of CTA pairs up to 1536, or 4096 with H up to 2560, CTA pairs on row tiles of
+ * 128 beyond) is chosen from B*L, H and V, and under stream capture from what the workspace holds; the environment variables
  * FDLLM_LMHEAD_GEMM (solo, pair, slab, wide) and FDLLM_LMHEAD_BN (256, 208) force one, for
  * measurements.
  * Results agree with fdllm_select applied to the fp32 logits fdllm_lmhead_logits writes

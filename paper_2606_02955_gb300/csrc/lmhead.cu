@@ -16,7 +16,7 @@
 //                            or CTA-pair (cta_group::2) variants
 //      lmhead_slab_kernel    (at most 32 rows) the operands swapped, W as the M = 128 side:
 //                            each CTA streams one vocabulary slab, one partial per row
-//      lmhead_wide_kernel    (up to 896 rows) the operands swapped on a CTA pair, W as the
+//      lmhead_wide_kernel    (up to 1536 or 4096 rows) the operands swapped on a CTA pair, W as the
 //                            M = 256 side and up to 256 (or 320) rows as N
 //   3. combine_rows_kernel   four warps per row fold its tile (or slab) partials in a fixed
 //                            order
@@ -770,8 +770,8 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
 // Here a stage is (128 + N / 2) x 128 B for 2 N cycles: 75 B/clock at N = 192, 58 at 320, and no
 // row tile is padded to 128.  LLaDA's head, 3/4 of B x 32 rows, whole fdllm_lmhead_confidence
 // pass, this variant against the better of solo and pair: B = 3 (72 rows) 160 against 163 us,
-// 8 165 against 190, 12 194 against 251, 16 244 against 261, 24 346 against 396, 28 385 against
-// 410, 32 426 against 422 and 64 795 against 785 (pair): the host takes it up to 28 x 32 rows.
+// 8 165 against 190, 12 194 against 251, 16 244 against 261, 24 338 against 397, 28 376 against
+// 405 (more rows at gemm_mode).
 // Other cuts measured: 288 rows in two blocks 220, in two groups of 160 instead of 160 and 128
 // 200 (back to back, at the power limit, 235 against 225), 381 rows in one block of two groups
 // 245, 480 rows in one block 311 against 293 in two.
@@ -877,7 +877,7 @@ struct WideItems {
     }
 };
 
-// Folds the states (M, S relative to M, first index) of one column from two sets of entries.  Either
+// Folds the states (M, S relative to M, first index) of one column from two sets of entries. Either
 // order gives the same bits.  -inf logits have S = 0; a NaN one leaves S NaN.
 __device__ __forceinline__ void wide_fold(float &M, float &S, uint32_t &I, float M2, float S2,
                                           uint32_t I2)
@@ -1658,12 +1658,26 @@ bool slab_preferred(int V)
     return slab_rows <= tile_rows;
 }
 
-// The GEMM variant: for at most kSlabRows rows the slab variant where slab_preferred, up to
-// kWideRowsMax rows the wide one, the pair beyond (both sides measured at lmhead_wide_kernel).
+// The GEMM variant: for at most kSlabRows rows the slab variant where slab_preferred, then the
+// wide one up to a number of rows, the pair beyond.  The pair computes whole tiles of 256 rows, and
+// with a short K loop (H up to kWideDeepH) its four epilogue warps set its pace: there the wide
+// variant stays ahead up to all the rows measured.  With a longer one it is level with the pair
+// at the rows of a whole tile and ahead in between, until the power limit decides (passes back to
+// back), where the pair needs less per row.  fdllm_lmhead_confidence, wide / pair, us:
+// H = 4096, V = 126464: of 32 x 32 rows 640 masked 368 / 398, 766 416 / 415; of 40 x 32 800 470 /
+// 507, 1280 654 / 656; of 48 x 32 1100 599 / 642, 1536 775 / 767 (back to back 888 / 869); of 64 x
+// 32 1300 695 / 740, 1478 773 / 760 (881 / 863), 2048 1021 / 1004; of 128 x 32 3000 1571 / 1514.
+// H = 3072, V = 80000: 1300 349 / 378, 2048 507 / 508, 4096 999 / 978.  H = 2048, V = 126464: 1300
+// 374 / 414, 1478 412 / 424, 2048 540 / 562, 4096 1064 / 1084.  H = 1024, V = 100000: 1478 194 /
+// 318, 4096 493 / 820.  H = 512, V = 30000: 2048 72 / 128.  fdllm_lmhead_logits, which takes the
+// same variant, H = 4096, V = 50000, 3/4 of 24 x 32 148 / 176, of 32 x 32 186 / 188, of 48 x 32 285
+// / 279; H = 1024, V = 30000, of 48 x 32 62 / 108.
 // FDLLM_LMHEAD_GEMM = solo, pair, slab or wide forces one (slab only where B * L <= kSlabRows).
-constexpr int kWideRowsMax = 28 * 32;
+constexpr int kWideDeepH = 2560;
+constexpr int kWideRowsMax = 4096;          // H <= kWideDeepH: the most rows measured
+constexpr int kWideRowsDeep = 48 * 32;      // H beyond
 
-int gemm_mode(int64_t rows, int V)
+int gemm_mode(int64_t rows, int H, int V)
 {
     if (const char *e = std::getenv("FDLLM_LMHEAD_GEMM")) {
         const std::string v(e);
@@ -1678,7 +1692,7 @@ int gemm_mode(int64_t rows, int V)
     }
     if (rows <= kSlabRows && slab_preferred(V))
         return kSlab;
-    return rows <= kWideRowsMax ? kWide : kPair;
+    return rows <= (H <= kWideDeepH ? kWideRowsMax : kWideRowsDeep) ? kWide : kPair;
 }
 
 int sm_count()
@@ -1865,7 +1879,7 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
                         float *conf = nullptr, int32_t *tok = nullptr)
 {
     const int64_t rows = (int64_t)B * L;
-    int mode = gemm_mode(rows, V);
+    int mode = gemm_mode(rows, H, V);
     int bn = 0, n_tiles = 0, w_tiles = 0;
     LmLayout lay;
     // partials per row: one per vocabulary tile (per CTA of the pair in the wide variant), or

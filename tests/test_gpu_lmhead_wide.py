@@ -28,8 +28,9 @@ SHAPES = [
     (5, 64, 128, 25000, 320),    # 98 tiles: a whole round, then a split one
     (6, 64, 136, 700, 321),      # two blocks of one group; a ragged K tail
     (9, 60, 64, 1000, 513),      # three blocks
-    (14, 64, 64, 3000, 896),     # the most rows that take this variant by default
-    (16, 66, 64, 3000, 1040),    # more
+    (14, 64, 64, 3000, 896),     # four blocks
+    (16, 66, 64, 3000, 1040),    # five
+    (128, 32, 64, 1500, 4096),   # sixteen: the most rows that take this variant by default
     (5, 64, 8, 20000, 320),      # H below one K-block
     (4, 64, 128, 19500, 225),    # 77 tiles: one left over, its group of 256 halved
     (4, 64, 64, 25000, 150),     # a group of 160 cut into 96 and 64
@@ -135,7 +136,9 @@ def test_capture_with_a_smaller_workspace(fd, monkeypatch):
     conf, tok = fd.fdllm_lmhead_confidence(h, w, m)
     fd.fdllm_release_workspace()
     big = torch.randn(33, 32, H, device="cuda").to(torch.bfloat16)
+    monkeypatch.setenv("FDLLM_LMHEAD_GEMM", "pair")
     fd.fdllm_lmhead_confidence(big, w, torch.ones((33, 32), dtype=torch.uint8, device="cuda"))
+    monkeypatch.delenv("FDLLM_LMHEAD_GEMM")
     c2, t2 = torch.zeros_like(conf), torch.zeros_like(tok)
     torch.cuda.synchronize()
     g = torch.cuda.CUDAGraph()
