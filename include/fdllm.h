@@ -35,10 +35,12 @@
  *     as FDLLM_ERR_NONFINITE.
  *   - All kernels are deterministic: the same inputs on the same GPU model give
  *     bit-identical outputs.  A position's confidence depends only on its logits and the
- *     call's shape (B * L, V, dtype), which fix how rows are cut into reduction units (in a
- *     workspace smaller than the shape's fdllm_workspace_bytes that still holds one partial
- *     per row, a row of at most 64 KB is one unit), so identical rows of one call give
- *     identical confidences (exact ties stay ties).
+ *     call's shape (B * L, V, dtype), which fix how rows are cut into reduction units, so
+ *     identical rows of one call give identical confidences (exact ties stay ties).  Only
+ *     where the workspace has no room for a shape's units (a caller's of fewer than
+ *     fdllm_workspace_bytes; the library's during a capture that no call of as large a shape
+ *     preceded) and yet for one per row is a row of at most 64 KB taken as one unit, with
+ *     other last bits.
  *   - Arithmetic: confidences are reduced in fp32 (relative error within 1e-5 of the exact
  *     value); the rules are evaluated on those fp32 confidences with exact 64-bit fixed-point
  *     prefix sums of 1 - c in units of 2^-52 (delta = 1 - f formed from the same integer as
@@ -102,16 +104,22 @@ typedef enum {
  *   out_n       [B] int32 device: number committed in each row; 0 iff the row had no
  *               masked position; FDLLM_ROW_NONFINITE / FDLLM_ROW_DEVICE_ERROR as above.
  *
- * The library's workspace is allocated on the current device at the first call that
- * needs more than it holds (cudaMalloc, which synchronises), then reused; make one call
- * of the largest shape before capturing the step in a CUDA graph.  Calls that share the
- * library workspace must be ordered on the GPU (one stream, or events); for concurrent
- * steps use fdllm_select_ws with a workspace per stream. */
+ * The library's workspace is allocated on the current device (cudaMalloc, which
+ * synchronises) by the first call of a larger shape than any before, then reused: after a
+ * call, no call of the same kind (from logits, or from hidden states of the LM head) with no
+ * larger B * L, row (V * sizeof(dtype)) and H allocates.  It does not grow during a stream
+ * capture: make one call of the largest shape before capturing the step in a CUDA graph.  A
+ * workspace that it outgrows is kept, for the graphs captured on it, until
+ * fdllm_release_workspace, and the next is at least twice as large where memory allows.  Calls
+ * that share the library workspace must be ordered on the GPU (one stream, or events); for
+ * concurrent steps use fdllm_select_ws with a workspace per stream. */
 fdllm_status fdllm_select(const void *logits, int dtype, int B, int L, int V, uint8_t *mask,
                           double param, int mode, int32_t *out_tokens, uint8_t *out_commit,
                           int32_t *out_n, void *stream);
 
-/* Bytes of caller workspace fdllm_select_ws needs for this shape (a pure host function). */
+/* Bytes of caller workspace fdllm_select_ws needs for this shape (a pure host function).  They do
+ * not always grow with the shape: a workspace for several shapes has the most that one of them
+ * needs. */
 size_t fdllm_workspace_bytes(int B, int L, int V, int dtype);
 
 /* fdllm_select with a caller-provided workspace (device, 256-byte aligned, at least
@@ -260,9 +268,11 @@ fdllm_status fdllm_select_host(const void *logits, int dtype, int B, int L, int 
  * bytes and a header), allocated outside the step as for fdllm_select.  Asynchronous on
  * `stream`.  The GEMM's tiling (vocabulary slabs for at most 32 rows, the vocabulary as the
  * wide operand of CTA pairs up to 1536, or 4096 with H up to 2560, CTA pairs on row tiles of
- * 128 beyond) is chosen from B*L, H and V, and under stream capture from what the workspace holds; the environment variables
- * FDLLM_LMHEAD_GEMM (solo, pair, slab, wide) and FDLLM_LMHEAD_BN (256, 208) force one, for
- * measurements.
+ * 128 beyond) is chosen from B*L, H and V; only during a capture that no call of as large a
+ * shape preceded may the workspace hold no more than the partials of row tiles, which then
+ * take the place of the wide operand.  For measurements the environment variable
+ * FDLLM_LMHEAD_GEMM (solo, pair, slab, wide) forces a tiling and FDLLM_LMHEAD_BN (256, 208) the
+ * vocabulary entries of a tile of solo and pair (it has no effect on the others).
  * Results agree with fdllm_select applied to the fp32 logits fdllm_lmhead_logits writes
  * under the same tiling (the same tensor-core accumulation): tokens bit-exact, confidences
  * within 1e-5. */
@@ -369,7 +379,7 @@ fdllm_status fdllm_profile_terms(const float *conf, const uint8_t *mask, int B, 
 fdllm_status fdllm_check_bounded_wait(double seconds, void *stream);
 
 /* Synchronises `stream`, then reports (and clears) the sticky device error of the library
- * workspace on the current device: FDLLM_ERR_DEVICE if a kernel gave up a bounded wait
+ * workspace (and of those it outgrew) on the current device: FDLLM_ERR_DEVICE if a kernel gave up a bounded wait
  * since the last call, else FDLLM_ERR_NONFINITE if a selection since the last call found a
  * row of FDLLM_ROW_NONFINITE, FDLLM_OK otherwise.  For fdllm_select_ws, pass the workspace to
  * fdllm_workspace_status instead.  Clearing an error also resets the workspace's work
@@ -378,7 +388,8 @@ fdllm_status fdllm_check_bounded_wait(double seconds, void *stream);
 fdllm_status fdllm_device_status(void *stream);
 fdllm_status fdllm_workspace_status(void *workspace, void *stream);
 
-/* Frees the library workspace of the current device (synchronises the device). */
+/* Frees the library workspace of the current device and those that it outgrew (synchronises the
+ * device): graphs captured on them must not be launched any more. */
 void fdllm_release_workspace(void);
 
 /* A static English description of a status code. */

@@ -2,9 +2,11 @@
 // the workspace (library-owned per device, or caller-provided) and the kernel launches.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <mutex>
+#include <vector>
 
 #include "fdllm.h"
 #include "fdllm_internal.cuh"
@@ -24,8 +26,35 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 //   partials UnitPartial [rows][units_per_row]
 struct Layout {
     size_t status, next_unit, partials, total;
+    size_t reserve;  // select_reserve_bytes of the call
     UnitPlan plan;
 };
+
+size_t scratch_bytes(int64_t partials)
+{
+    return align_up(kAlign + (size_t)partials * sizeof(UnitPartial));
+}
+
+}  // namespace
+
+// The need of a call falls in places as its shape grows: short rows take more partials than long
+// ones, a small step takes more units per row than a large one.
+size_t select_reserve_bytes(int64_t rows, int64_t row_bytes)
+{
+    auto units = [](int64_t bytes, int64_t target) { return (bytes + target - 1) / target; };
+    const int64_t large = rows * units(row_bytes, kUnitTargetBytes);
+    // rows * row_bytes <= kSmallStepBytes bounds the units of a small step, one more per row for
+    // the part that does not fill one
+    const int64_t small = std::min(rows * units(row_bytes, kSmallUnitTargetBytes),
+                                   kSmallStepBytes / kSmallUnitTargetBytes + rows);
+    int64_t warp = 0;
+    if (rows > kWarpMinRows)
+        warp = std::min(rows * units(std::min(row_bytes, kWarpRowBytes), kWarpUnitVecs * 16),
+                        std::max(rows, kMostWarpUnits));
+    return scratch_bytes(std::max({large, small, warp}));
+}
+
+namespace {
 
 Layout layout_for(int64_t rows, int64_t row_bytes, bool warp_units = true)
 {
@@ -34,7 +63,8 @@ Layout layout_for(int64_t rows, int64_t row_bytes, bool warp_units = true)
     l.status = 0;
     l.next_unit = 4;
     l.partials = kAlign;
-    l.total = align_up(l.partials + (size_t)rows * l.plan.units_per_row * sizeof(UnitPartial));
+    l.total = scratch_bytes(rows * l.plan.units_per_row);
+    l.reserve = select_reserve_bytes(rows, row_bytes);
     return l;
 }
 
@@ -79,42 +109,65 @@ fdllm_status check_logits(const void *logits, int dtype, int V)
     return FDLLM_OK;
 }
 
-// Library-owned workspace, one per device, grown on demand and zero-filled when allocated.
+// Library-owned workspace, one per device, grown on demand and zero-filled when allocated.  A graph
+// captured earlier may hold the buffer that the workspace outgrows, so that one is kept until
+// fdllm_release_workspace.  The next is at least twice as large where memory allows, so all that is
+// kept is less than the workspace itself.
 struct OwnedWorkspace {
     void *ptr = nullptr;
     size_t bytes = 0;
+    std::vector<void *> kept;
 };
 constexpr int kMaxDevices = 64;
 OwnedWorkspace g_ws[kMaxDevices];
 std::mutex g_ws_mutex;
 
+bool is_capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return cap != cudaStreamCaptureStatusNone;
+}
+
+// A zero-filled buffer of `want` bytes, or of `least` where there is no room for that.
+fdllm_status grow(OwnedWorkspace &w, size_t least, size_t want, cudaStream_t stream)
+{
+    void *p = nullptr;
+    size_t bytes = want;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+        (void)cudaGetLastError();
+        bytes = least;
+        if (least == want || cudaMalloc(&p, bytes) != cudaSuccess)
+            return FDLLM_ERR_CUDA;
+    }
+    if (cudaMemsetAsync(p, 0, bytes, stream) != cudaSuccess) {
+        cudaFree(p);
+        return FDLLM_ERR_CUDA;
+    }
+    if (w.ptr)
+        w.kept.push_back(w.ptr);
+    w.ptr = p;
+    w.bytes = bytes;
+    return FDLLM_OK;
+}
+
 }  // namespace
 
-fdllm_status owned_workspace(size_t need, cudaStream_t stream, void **out)
+fdllm_status owned_workspace(size_t need, size_t reserve, cudaStream_t stream, void **out)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
         return FDLLM_ERR_CUDA;
     std::lock_guard<std::mutex> lock(g_ws_mutex);
     OwnedWorkspace &w = g_ws[dev];
-    if (w.bytes < need) {
-        if (w.ptr) {
-            if (cudaDeviceSynchronize() != cudaSuccess)
-                return FDLLM_ERR_CUDA;
-            cudaFree(w.ptr);
-            w.ptr = nullptr;
-            w.bytes = 0;
-        }
-        void *p = nullptr;
-        if (cudaMalloc(&p, need) != cudaSuccess)
-            return FDLLM_ERR_CUDA;
-        if (cudaMemsetAsync(p, 0, need, stream) != cudaSuccess) {
-            cudaFree(p);
-            return FDLLM_ERR_CUDA;
-        }
-        w.ptr = p;
-        w.bytes = need;
-    }
+    reserve = std::max(need, reserve);
+    if (w.bytes < reserve && !(w.ptr && is_capturing(stream)))
+        (void)grow(w, reserve, std::max(reserve, 2 * w.bytes), stream);
+    if (w.bytes < need)
+        return FDLLM_ERR_CUDA;
     *out = w.ptr;
     return FDLLM_OK;
 }
@@ -134,11 +187,7 @@ size_t owned_bytes()
 
 bool owned_workspace_ready(size_t need, cudaStream_t stream)
 {
-    if (need <= owned_bytes())
-        return true;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(stream, &cap) != cudaSuccess ||
-           cap == cudaStreamCaptureStatusNone;
+    return need <= owned_bytes() || !is_capturing(stream);
 }
 
 namespace {
@@ -288,7 +337,7 @@ fdllm_status select_owned(const void *logits, int dtype, int B, int L, int V, ui
         return st;
     const Layout lay = owned_layout((int64_t)B * L, (int64_t)V * esize_of(dtype), stream);
     void *ws = nullptr;
-    st = owned_workspace(lay.total, stream, &ws);
+    st = owned_workspace(lay.total, lay.reserve, stream, &ws);
     if (st != FDLLM_OK)
         return st;
     return run_select(logits, dtype, B, L, V, mask, param, mode, out_tokens, out_commit, out_n,
@@ -349,7 +398,7 @@ fdllm_status fdllm_select_robust(const void *logits, int dtype, int B, int L, in
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const Layout lay = owned_layout((int64_t)B * L, (int64_t)V * esize_of(dtype), s);
     void *ws = nullptr;
-    st = owned_workspace(lay.total, s, &ws);
+    st = owned_workspace(lay.total, lay.reserve, s, &ws);
     if (st != FDLLM_OK)
         return st;
     return run_select(logits, dtype, B, L, V, mask, param, kModeRobust, out_tokens, out_commit,
@@ -397,7 +446,7 @@ fdllm_status fdllm_confidence(const void *logits, int dtype, int B, int L, int V
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const Layout lay = owned_layout((int64_t)B * L, (int64_t)V * esize_of(dtype), s);
     void *ws = nullptr;
-    st = owned_workspace(lay.total, s, &ws);
+    st = owned_workspace(lay.total, lay.reserve, s, &ws);
     if (st != FDLLM_OK)
         return st;
     VocabReduceArgs ra = reduce_args(logits, dtype, B, L, V, mask, static_cast<uint8_t *>(ws),
@@ -434,7 +483,7 @@ fdllm_status fdllm_vocab_reduce(const void *logits, int dtype, int B, int L, int
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const Layout lay = owned_layout((int64_t)B * L, (int64_t)V * esize_of(dtype), s);
     void *ws = nullptr;
-    st = owned_workspace(lay.total, s, &ws);
+    st = owned_workspace(lay.total, lay.reserve, s, &ws);
     if (st != FDLLM_OK)
         return st;
     VocabReduceArgs ra = reduce_args(logits, dtype, B, L, V, mask, static_cast<uint8_t *>(ws),
@@ -519,15 +568,22 @@ fdllm_status fdllm_device_status(void *stream)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
         return FDLLM_ERR_CUDA;
-    void *ptr = nullptr;
+    std::vector<void *> buffers;  // graphs captured before the workspace grew use the kept ones
     {
         std::lock_guard<std::mutex> lock(g_ws_mutex);
-        ptr = g_ws[dev].ptr;
+        buffers = g_ws[dev].kept;
+        if (g_ws[dev].ptr)
+            buffers.push_back(g_ws[dev].ptr);
     }
-    if (!ptr)
-        return FDLLM_OK;
-    return read_and_clear_status(static_cast<uint32_t *>(ptr), static_cast<cudaStream_t>(stream),
-                                 kHeaderClearBytes);
+    fdllm_status worst = FDLLM_OK;  // a gave-up wait outranks a non-finite row
+    for (void *p : buffers) {
+        const fdllm_status st = read_and_clear_status(
+            static_cast<uint32_t *>(p), static_cast<cudaStream_t>(stream), kHeaderClearBytes);
+        if (st == FDLLM_ERR_CUDA)
+            return st;
+        worst = std::max(worst, st);
+    }
+    return worst;
 }
 
 fdllm_status fdllm_workspace_status(void *workspace, void *stream)
@@ -557,8 +613,9 @@ void fdllm_release_workspace(void)
     if (g_ws[dev].ptr) {
         cudaDeviceSynchronize();
         cudaFree(g_ws[dev].ptr);
-        g_ws[dev].ptr = nullptr;
-        g_ws[dev].bytes = 0;
+        for (void *p : g_ws[dev].kept)
+            cudaFree(p);
+        g_ws[dev] = OwnedWorkspace();
     }
     release_host_staging(dev);
 }

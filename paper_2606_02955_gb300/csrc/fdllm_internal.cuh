@@ -83,6 +83,9 @@ constexpr int64_t kWarpRowBytes = 65536;
 constexpr int64_t kWarpMinRows = 2 * 152;
 constexpr int64_t kWarpUnitVecs = 512;
 static_assert(kWarpRowBytes / 16 / kWarpUnitVecs <= 8, "partials folded in one round");
+// Beyond one per row, no more warp units than the static scratch array has room for.
+constexpr int64_t kMostWarpUnits =
+    (FDLLM_STATIC_SCRATCH_BYTES - 256) / (int64_t)sizeof(UnitPartial);
 
 // warp_units = false plans CTA units whatever the shape: one partial per short row, for scratch
 // memory that does not hold more (see layout_within).
@@ -90,9 +93,7 @@ inline UnitPlan plan_units(int64_t row_bytes, int64_t rows, bool warp_units = tr
 {
     const int64_t vpr = row_bytes / 16;
     if (warp_units && row_bytes <= kWarpRowBytes && rows > kWarpMinRows) {
-        // no more units than the static scratch array has room for
-        const int64_t fit =
-            (FDLLM_STATIC_SCRATCH_BYTES - 256) / (int64_t)sizeof(UnitPartial) / rows;
+        const int64_t fit = kMostWarpUnits / rows;
         int64_t upr = (vpr + kWarpUnitVecs - 1) / kWarpUnitVecs;
         upr = upr > fit ? fit : upr;
         upr = upr < 1 ? 1 : upr;
@@ -172,15 +173,23 @@ fdllm_status lmhead_select_owned(const void *hidden, const void *w_vocab, int B,
                                  int32_t *out_tokens, uint8_t *out_commit, int32_t *out_n,
                                  cudaStream_t stream, bool pdl);
 
-// The library-owned workspace of the current device, grown on demand and zero-filled when
-// allocated.  Every user shares its 256-byte header: the sticky status word at offset 0 and
-// the vocab reduction's work counter at 4 (zero between calls); the LM-head path keeps its
-// compact row count at 8.
-fdllm_status owned_workspace(size_t need, cudaStream_t stream, void **out);
+// The library-owned workspace of the current device, at least `need` bytes.  Outside a capture it
+// is grown to `reserve`, the most that any call of no larger a shape needs (where memory allows:
+// a call goes on with `need`), and zero-filled when allocated; during one it stays as it is.
+// Every user shares its 256-byte header: the sticky status word at offset 0 and the vocab
+// reduction's work counter at 4 (zero between calls); the LM-head path keeps its compact row
+// count at 8.
+fdllm_status owned_workspace(size_t need, size_t reserve, cudaStream_t stream, void **out);
 
 // Whether owned_workspace can give `need` bytes: the workspace holds them, or `stream` is not
-// being captured (the workspace cannot grow during a capture).
+// being captured (the workspace does not grow during a capture).
 bool owned_workspace_ready(size_t need, cudaStream_t stream);
+
+// The most workspace that any selection of no more and no longer rows needs; the need of an LM-head
+// call, and the most of any with no more rows, no larger a hidden size and no longer a vocabulary.
+size_t select_reserve_bytes(int64_t rows, int64_t row_bytes);
+size_t lmhead_need_bytes(int64_t rows, int H, int V);
+size_t lmhead_reserve_bytes(int64_t rows, int H, int V);
 
 // fdllm_select's argument checks (shape, pointers, mode, param, logits alignment and the
 // unit plan's index range), done before anything is enqueued.

@@ -24,6 +24,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdlib>
@@ -1871,6 +1872,30 @@ cudaError_t launch_gemm(const CUtensorMap &mh, const CUtensorMap &mw, const Gemm
     }
 }
 
+// How one call is cut, and its workspace.
+struct LmPlan {
+    int mode, bn;  // bn: W rows of a tile (per CTA in the wide variant)
+    int w_tiles;   // tiles of 2 bn W rows
+    int n_tiles;   // partials per row: one per vocabulary tile (per CTA of the pair in the wide
+                   // variant), or one per CTA of the slab variant
+    LmLayout lay;
+};
+
+LmPlan lm_plan(int mode, int64_t rows, int H, int V)
+{
+    LmPlan p;
+    p.mode = mode;
+    p.bn = mode == kSlab   ? slab_height(V)
+           : mode == kWide ? wide_height(rows, V)
+                           : choose_bn(rows, V, mode == kPair);
+    p.w_tiles = (V + 2 * p.bn - 1) / (2 * p.bn);
+    p.n_tiles = mode == kSlab   ? slab_grid(V)
+                : mode == kWide ? 2 * p.w_tiles
+                                : (V + p.bn - 1) / p.bn;
+    p.lay = lm_layout(rows, H, p.n_tiles);
+    return p;
+}
+
 // Steps 1-2 (and 3 for the reduce epilogue) on the owned workspace.  The confidences and
 // argmaxes go to conf and tok [B, L], or to the workspace where those are null.
 fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, int V,
@@ -1879,30 +1904,15 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
                         float *conf = nullptr, int32_t *tok = nullptr)
 {
     const int64_t rows = (int64_t)B * L;
-    int mode = gemm_mode(rows, H, V);
-    int bn = 0, n_tiles = 0, w_tiles = 0;
-    LmLayout lay;
-    // partials per row: one per vocabulary tile (per CTA of the pair in the wide variant), or
-    // one per CTA of the slab variant
-    auto plan = [&] {
-        bn = mode == kSlab   ? slab_height(V)
-             : mode == kWide ? wide_height(rows, V)
-                             : choose_bn(rows, V, mode == kPair);
-        w_tiles = (V + 2 * bn - 1) / (2 * bn);
-        n_tiles = mode == kSlab   ? slab_grid(V)
-                  : mode == kWide ? 2 * w_tiles
-                                  : (V + bn - 1) / bn;
-        lay = lm_layout(rows, H, n_tiles);
-    };
-    plan();
-    // Under capture the workspace cannot grow; one left by larger calls of the tile variants,
-    // whose partials are fewer, may hold only those.
-    if (mode == kWide && !owned_workspace_ready(lay.total, s)) {
-        mode = (rows + BM - 1) / BM >= 8 ? kPair : kSolo;
-        plan();
-    }
+    LmPlan plan = lm_plan(gemm_mode(rows, H, V), rows, H, V);
+    // The workspace does not grow under capture; one that calls of other shapes have sized may hold
+    // only the tile variants' partials, which are fewer.
+    if (plan.mode == kWide && !owned_workspace_ready(plan.lay.total, s))
+        plan = lm_plan((rows + BM - 1) / BM >= 8 ? kPair : kSolo, rows, H, V);
+    const int mode = plan.mode, bn = plan.bn, n_tiles = plan.n_tiles;
+    const LmLayout lay = plan.lay;
     void *wsv = nullptr;
-    fdllm_status st = owned_workspace(lay.total, s, &wsv);
+    fdllm_status st = owned_workspace(lay.total, lmhead_reserve_bytes(rows, H, V), s, &wsv);
     if (st != FDLLM_OK)
         return st;
     uint8_t *ws = static_cast<uint8_t *>(wsv);
@@ -1944,7 +1954,7 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
     g.k_blocks = (H + BK - 1) / BK;
     g.slab_h = mode == kSlab ? bn : 0;
     g.slab_tiles = mode == kSlab ? (V + bn - 1) / bn : 0;
-    g.w_tiles = w_tiles;
+    g.w_tiles = plan.w_tiles;
     g.wide_h = mode == kWide ? bn : 0;
     g.partials = reinterpret_cast<UnitPartial *>(ws + lay.partials);
     g.logits = out_logits;
@@ -1980,6 +1990,23 @@ fdllm_status run_lmhead(const void *hidden, const void *w, int B, int L, int H, 
 using namespace fdllm;
 
 namespace fdllm {
+
+size_t lmhead_need_bytes(int64_t rows, int H, int V)
+{
+    return lm_plan(gemm_mode(rows, H, V), rows, H, V).lay.total;
+}
+
+// The wide variant keeps up to twice the pair's partials per row, lower tiles more again, and how
+// far up it serves depends on H: the need of a call falls in places as its shape grows.
+size_t lmhead_reserve_bytes(int64_t rows, int H, int V)
+{
+    auto bytes = [](int64_t r, int h, int64_t n_tiles) { return lm_layout(r, h, n_tiles).total; };
+    const int64_t wide = 2 * (((int64_t)V + 255) / 256);
+    return std::max({bytes(rows, H, ((int64_t)V + 207) / 208),
+                     bytes(std::min<int64_t>(rows, kWideLowRows), H, 2 * (((int64_t)V + 191) / 192)),
+                     bytes(std::min<int64_t>(rows, kWideRowsDeep), H, wide),
+                     bytes(std::min<int64_t>(rows, kWideRowsMax), std::min(H, kWideDeepH), wide)});
+}
 
 fdllm_status lmhead_select_owned(const void *hidden, const void *w_vocab, int B, int L, int H,
                                  int V, uint8_t *mask, double param, int mode,

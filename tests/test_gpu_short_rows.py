@@ -113,10 +113,11 @@ def test_scratch_of_one_partial_per_row_serves(fd, orc):
     with pytest.raises(fd.FdllmError) as e:
         fd.fdllm_select_ws(x, mask, 0.75, "profile", ws[:256 + 320 * 16 - 256])
     assert e.value.status == 5
-    # the library's workspace as a longer vocabulary left it, then a capture
+    # the library's workspace as fewer rows (no warp units) of a longer vocabulary left it, then a
+    # capture
     fd.fdllm_release_workspace()
-    fd.fdllm_select(torch.randn(10, 32, 8 * 8000, device="cuda").to(torch.bfloat16),
-                    torch.ones((10, 32), dtype=torch.uint8, device="cuda"), 0.75)
+    fd.fdllm_select(torch.randn(8, 38, 8 * 8000, device="cuda").to(torch.bfloat16),
+                    torch.ones((8, 38), dtype=torch.uint8, device="cuda"), 0.75)
     out = (torch.full((10, 32), -1, dtype=torch.int32, device="cuda"),
            torch.zeros((10, 32), dtype=torch.uint8, device="cuda"),
            torch.zeros((10,), dtype=torch.int32, device="cuda"))
