@@ -243,9 +243,11 @@ fdllm_status fdllm_gather_masked_rows(const void *src, void *dst, int dtype, int
  * place when the call returns.  Where out_tokens, out_commit and out_n are page-locked and
  * the mask is in host memory, the step writes the three over the host link and the host
  * clears the committed positions of the mask after the synchronisation; otherwise out_tokens
- * is staged as well, and all four are copied back.  Argument errors are reported before
- * anything is enqueued; the same device errors as fdllm_select (fdllm_device_status).  Not
- * for stream capture (it synchronises).
+ * is staged as well, and all four are copied back.  An array of which only a part is page-locked
+ * is refused (FDLLM_ERR_CUDA: the runtime does not copy such a range).  Argument errors are reported before
+ * anything is enqueued; the same device errors as fdllm_select (fdllm_device_status).  A call
+ * that returns FDLLM_ERR_CUDA may have written page-locked results in part, and then leaves
+ * the mask as it was.  Not for stream capture (it synchronises).
  * Calls share the staging buffer and the library workspace of their device: calls from
  * several host threads at once must be serialised by the caller.  The paper has no
  * counterpart. */

@@ -3,6 +3,7 @@
 // so that only the logits the selection needs cross the link; fdllm_select_host wraps that,
 // the step and the copies of its results back to the host in one call.
 #include <cuda_runtime.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <cstdint>
@@ -10,6 +11,7 @@
 
 #include "fdllm.h"
 #include "fdllm_internal.cuh"
+#include "host_view.h"
 
 namespace fdllm {
 namespace {
@@ -68,20 +70,22 @@ const void *device_view(const void *src)
 }
 
 // The mapping through which the GPU writes n elements of page-locked host memory; nullptr for any
-// other memory and where the end of the array is not mapped with its beginning.
+// other memory and where a part of the array is not mapped.
 template <typename T>
 T *pinned_view(T *p, int64_t n)
 {
-    cudaPointerAttributes first, last;
-    if (cudaPointerGetAttributes(&first, p) != cudaSuccess ||
-        cudaPointerGetAttributes(&last, p + n - 1) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return nullptr;
-    }
-    if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost)
-        return nullptr;
-    T *const d = static_cast<T *>(first.devicePointer);
-    return d && d + n - 1 == static_cast<T *>(last.devicePointer) ? d : nullptr;
+    static const int64_t page = sysconf(_SC_PAGESIZE);
+    auto device_of = [](uint8_t *host) -> uint8_t * {
+        cudaPointerAttributes attr;
+        if (cudaPointerGetAttributes(&attr, host) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return nullptr;
+        }
+        return attr.type == cudaMemoryTypeHost ? static_cast<uint8_t *>(attr.devicePointer)
+                                               : nullptr;
+    };
+    return reinterpret_cast<T *>(whole_view(reinterpret_cast<uint8_t *>(p),
+                                            n * (int64_t)sizeof(T), page, device_of));
 }
 
 // Whether the host itself reads and writes p (pageable or page-locked memory).
