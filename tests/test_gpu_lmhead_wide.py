@@ -53,27 +53,62 @@ def drawn(B, L, H, V, rows):
     return h, w, mask
 
 
-@pytest.mark.parametrize("B,L,H,V,rows", SHAPES)
-def test_gemm_and_reduction(fd, orc, wide, B, L, H, V, rows):
-    """The stored accumulators within the fp32 bound of the exact products, and the fused
-    confidences those of the same accumulators."""
-    h, w, mask = drawn(B, L, H, V, rows)
+def check_gemm_and_reduction(fd, orc, h, w, mask, entries=None):
+    """The stored accumulators (at the given vocabulary entries) within the fp32 bound of the exact
+    products, and the fused confidences those of the same accumulators."""
     m = torch.from_numpy(mask).cuda()
     x = fd.fdllm_lmhead_logits(h, w, m)
     conf, tok = fd.fdllm_lmhead_confidence(h, w, m)
     assert fd.fdllm_device_status() == 0
     mk = mask.astype(bool)
     xg = x.cpu().numpy()
-    ref, mag = orc.lmhead_logits(bits(h), bits(w), mask=mask, with_abs=True,
-                                 nthreads=oracle_threads())
-    err = np.abs(xg[mk].astype(np.float64) - ref[mk])
-    assert (err <= gemm_bound(mag[mk], ref[mk], H)).all(), err.max()
+    at = np.arange(w.shape[0]) if entries is None else entries
+    ref, mag = orc.lmhead_logits(bits(h), bits(w[torch.from_numpy(at).cuda()]), mask=mask,
+                                 with_abs=True, nthreads=oracle_threads())
+    err = np.abs(xg[mk][:, at].astype(np.float64) - ref[mk])
+    assert (err <= gemm_bound(mag[mk], ref[mk], h.shape[-1])).all(), err.max()
     assert np.isnan(xg[~mk]).all()
     rc, rt, bad = orc.confidence(np.nan_to_num(xg, nan=0.0), mask, nthreads=oracle_threads())
     assert bad == 0
     assert np.array_equal(tok.cpu().numpy()[mk], rt[mk])
     c = conf.cpu().numpy().astype(np.float64)
     assert (np.abs(c[mk] - rc[mk]) / rc[mk]).max() <= CONF_RTOL
+
+
+@pytest.mark.parametrize("B,L,H,V,rows", SHAPES)
+def test_gemm_and_reduction(fd, orc, wide, B, L, H, V, rows):
+    check_gemm_and_reduction(fd, orc, *drawn(B, L, H, V, rows))
+
+
+# K loops longer than the ring (at most 11 stages of 64): stages reused within an item, and with two
+# groups the first one held up by a full ring while the second one's accumulator is being read
+LONG = [
+    (10, 32, 1024, 45000, 288),  # groups of 160 and 128: two rounds of W tiles, then split ones
+    (10, 32, 1024, 45000, 320),  # two groups of 160
+    (10, 32, 4096, 25000, 288),  # a round, then tiles split between the groups
+    (10, 32, 4096, 25000, 320),
+    (8, 32, 4096, 25000, 200),   # one group, the tiles left over halved
+    (9, 32, 4096, 20000, 257),   # two groups: 79 tiles
+    (8, 32, 4096, 45000, 256),   # one group of 256
+]
+
+
+@pytest.mark.parametrize("B,L,H,V,rows", LONG)
+def test_long_hidden_size(fd, orc, wide, B, L, H, V, rows):
+    """Logits checked at the first and last entries and at drawn ones (every W tile among them)."""
+    rng = np.random.default_rng(H + rows)
+    at = np.concatenate([np.arange(300), np.arange(V - 300, V), np.arange(300, V - 300, 37),
+                         rng.integers(0, V, 200)])
+    check_gemm_and_reduction(fd, orc, *drawn(B, L, H, V, rows), entries=np.unique(at))
+
+
+@pytest.mark.parametrize("B,L,H,V", [(48, 32, 2568, 600), (29, 53, 2568, 600),
+                                     (64, 64, 2560, 300), (17, 241, 2560, 300)])
+def test_either_side_of_the_choice(fd, orc, monkeypatch, B, L, H, V):
+    """1536 and 1537 rows of H beyond 2560, 4096 and 4097 of H up to it, by the host's own choice."""
+    monkeypatch.delenv("FDLLM_LMHEAD_GEMM", raising=False)
+    monkeypatch.delenv("FDLLM_LMHEAD_BN", raising=False)
+    check_gemm_and_reduction(fd, orc, *drawn(B, L, H, V, B * L - 3))
 
 
 @pytest.mark.parametrize("k", [12, 26, 122])
