@@ -1597,7 +1597,6 @@ fdllm_status check_lmhead(const void *hidden, const void *w, int B, int L, int H
 }
 
 int sm_count();
-int choose_bn(int64_t rows, int V, bool pair);
 
 // The slab variant's tile height: the multiple of 8 in [96, 128] that minimises the W rows
 // of the busiest CTA, ceil(ceil(V / h) / P) * h with P = min(tiles, SMs); ties go to the
@@ -1642,25 +1641,10 @@ int slab_grid(int V)
     return (int)(tiles < sm_count() ? tiles : sm_count());
 }
 
-// Rows of W per CTA on the longest-running SM, for the slab variant (whole tiles of its
-// height) against the tile variant (one row tile: whole waves of vocabulary tiles times
-// their width).  The slab variant's row operand is 4 KB per K-block where a row tile's is
-// 16 KB, so more of each stage is W; measured on LLaDA-sized heads, it is faster when its
-// busiest CTA streams no more rows.
-bool slab_preferred(int V)
-{
-    const int64_t sms = sm_count();
-    const int64_t h = slab_height(V);
-    const int64_t tiles = ((int64_t)V + h - 1) / h;
-    const int64_t P = tiles < sms ? tiles : sms;
-    const int64_t slab_rows = (tiles + P - 1) / P * h;
-    const int bn = choose_bn(1, V, false);
-    const int64_t tile_rows = ((V + bn - 1) / bn + sms - 1) / sms * bn;
-    return slab_rows <= tile_rows;
-}
-
-// The GEMM variant: for at most kSlabRows rows the slab variant where slab_preferred, then the
-// wide one up to a number of rows, the pair beyond.  The pair computes whole tiles of 256 rows, and
+// The GEMM variant: the slab variant for at most kSlabRows rows (its row operand is 4 KB per K-block
+// where a row tile's is 16 KB, and its busiest CTA never streams more W rows than with row tiles,
+// since half of either tile width is one of its heights), then the wide one up to a number of rows,
+// the pair beyond.  The pair computes whole tiles of 256 rows, and
 // with a short K loop (H up to kWideDeepH) its four epilogue warps set its pace: there the wide
 // variant stays ahead up to all the rows measured.  With a longer one it is level with the pair
 // at the rows of a whole tile and ahead in between, until the power limit decides (passes back to
@@ -1691,7 +1675,7 @@ int gemm_mode(int64_t rows, int H, int V)
         if (v == "wide")
             return kWide;
     }
-    if (rows <= kSlabRows && slab_preferred(V))
+    if (rows <= kSlabRows)
         return kSlab;
     return rows <= (H <= kWideDeepH ? kWideRowsMax : kWideRowsDeep) ? kWide : kPair;
 }
