@@ -827,11 +827,12 @@ struct WidePiece {
 
 // The pieces of one CTA pair.  Whole rounds of items over the pairs first; if what is left then
 // fills at most half of them, each leftover item goes to two pairs, one group or half of the one
-// group each.  Halves of fewer than 80 columns would gain nothing, since a stage's W share alone
-// takes as long to arrive as 128 columns' MMAs.  Whole fdllm_lmhead_confidence pass with one-group
-// items left whole against halved: 200 rows, H = 4096, 20000 entries 49.5 -> 46.4 us, 65000 entries
-// 98.7 -> 95.8, LLaDA's 169 -> 167; H = 1024, 20000 entries 200 rows 20.6 -> 19.5, 700 rows 32.9 ->
-// 31.4; H = 2048, 8000 entries 200 rows 19.5 -> 17.5.
+// group each: halves of 96 and 64 columns (a group of 160) and up, since no narrower group was tried.
+// Whole fdllm_lmhead_confidence pass with one-group items left whole against halved: 200 rows, H =
+// 4096, 20000 entries 49.5 -> 46.4 us, 65000 entries 98.7 -> 95.8, LLaDA's 169 -> 167; H = 1024,
+// 20000 entries 200 rows 20.6 -> 19.5, 700 rows 32.9 -> 31.4; H = 2048, 8000 entries 200 rows 19.5
+// -> 17.5.  In a group of 160: 144 rows, H = 1024, 20000 entries 19.3 -> 18.1, H = 4096, 25000
+// entries 48.2 -> 47.5, LLaDA's 162.2 -> 161.8; 160 rows, H = 2048, 45000 entries 42.5 -> 41.6.
 constexpr int kWideHalved = 160;
 
 struct WideItems {
@@ -1335,10 +1336,10 @@ __global__ void __launch_bounds__(kPackThreads)
 }
 
 // The pair variant's rows are packed by two kernels, this list and a copy by one small CTA per row,
-// although that takes 2 us longer: the GEMM's clusters are then placed while 2048 such CTAs come
-// and go, mostly one die of the GPU first, and the six pairs that share a W tile mostly share its
-// L2.  Behind pack_rows_kernel they end up mixed, which costs more than 2 us of the power that
-// limits this variant: 64 x 32 rows back to back 891 against 902 us (clusters in SM order 903).
+// although that takes 2 us longer: 64 x 32 rows back to back, where the board's power limits this
+// variant, take 891 us behind them and 902 behind pack_rows_kernel.  Measured, not explained: the
+// GEMM's clusters land on the SMs in another order while 2048 such CTAs come and go, perhaps one
+// that shares W tiles better between the two dies (clusters handed out in SM order: 903).
 //
 // One CTA: the packed list of masked rows (ascending) and its length.
 __global__ void __launch_bounds__(1024) compact_rows_kernel(const uint8_t *mask, int rows,
@@ -1623,9 +1624,11 @@ int slab_height(int V)
 // variant's heights (104 for LLaDA's V: eight whole rounds instead of six and a half) balance
 // that: of 128 rows 8 masked 155 against 163 us, 32 157 against 163, 96 158 against 159, 128 160
 // against 160.  More rows make it the tensor cores', whose M = 256 a lower tile leaves partly
-// unused: of 192 rows all masked 167 against 164, of 256 190 against 178 (but 16 of them 157
-// against 163), 288 of 384 229 against 195.  So the line lies at 192, by the shape alone: a row's
-// partials must not depend on how many rows are masked.
+// unused: of 192 rows all masked 167 against 164, of 256 196 against 178, 288 of 384 225 against
+// 195.  So the line lies at 192, by the shape alone: a row's partials must not depend on how many
+// rows are masked, and so beyond it a few masked rows take the tall tiles, too (of 256 rows 16
+// masked 156 low, 162 tall, 64 157 and 160; with row tiles 158 against 157 tall on another box).
+// Measured on LLaDA's V; at V = 50000, H = 4096 256 of 256 rows are level (79 low, 81 tall).
 constexpr int kWideLowRows = 192;
 
 int wide_height(int64_t rows, int V)
@@ -1645,21 +1648,26 @@ int slab_grid(int V)
 // where a row tile's is 16 KB, and its busiest CTA never streams more W rows than with row tiles,
 // since half of either tile width is one of its heights), then the wide one up to a number of rows,
 // the pair beyond.  The pair computes whole tiles of 256 rows, and
-// with a short K loop (H up to kWideDeepH) its four epilogue warps set its pace: there the wide
-// variant stays ahead up to all the rows measured.  With a longer one it is level with the pair
-// at the rows of a whole tile and ahead in between, until the power limit decides (passes back to
-// back), where the pair needs less per row.  fdllm_lmhead_confidence, wide / pair, us:
-// H = 4096, V = 126464: of 32 x 32 rows 640 masked 368 / 398, 766 416 / 415; of 40 x 32 800 470 /
-// 507, 1280 654 / 656; of 48 x 32 1100 599 / 642, 1536 775 / 767 (back to back 888 / 869); of 64 x
-// 32 1300 695 / 740, 1478 773 / 760 (881 / 863), 2048 1021 / 1004; of 128 x 32 3000 1571 / 1514.
-// H = 3072, V = 80000: 1300 349 / 378, 2048 507 / 508, 4096 999 / 978.  H = 2048, V = 126464: 1300
-// 374 / 414, 1478 412 / 424, 2048 540 / 562, 4096 1064 / 1084.  H = 1024, V = 100000: 1478 194 /
-// 318, 4096 493 / 820.  H = 512, V = 30000: 2048 72 / 128.  fdllm_lmhead_logits, which takes the
-// same variant, H = 4096, V = 50000, 3/4 of 24 x 32 148 / 176, of 32 x 32 186 / 188, of 48 x 32 285
-// / 279; H = 1024, V = 30000, of 48 x 32 62 / 108.
+// with a short K loop (H up to 2048) its four epilogue warps set its pace: there the wide variant
+// stays ahead up to all the rows measured.  With a longer one it is level with the pair at the rows
+// of a whole tile and ahead in between and with few rows masked, until the power limit decides
+// (passes back to back), where the pair needs 1 to 3 % less.  fdllm_lmhead_confidence, wide / pair,
+// us (back to back in brackets):
+// H = 4096, V = 126464: of 32 x 32 rows 51 masked 160 / 182, 640 368 / 398, 768 431 / 426 (494 /
+// 484); of 40 x 32 640 383 / 413, 800 470 / 507, 1280 684 / 683 (775 / 775); of 48 x 32 76 159 /
+// 188, 768 428 / 425, 1100 599 / 642, 1536 808 / 797 (920 / 902); of 64 x 32 102 161 / 189, 1300
+// 695 / 740, 1536 813 / 793 (928 / 900), 2048 1070 / 1043; of 96 x 32 3072 1611 / 1535.
+// H = 3072, V = 80000: of 1536 1152 334 / 335 (380 / 377); of 2048 102 90 / 106, 2048 512 / 514.
+// H = 2560, V = 126464: of 2048 102 106 / 125, 1024 353 / 352, 2048 675 / 671 (767 / 762); of 4096
+// 204 114 / 130, 2048 683 / 675, 4096 1346 / 1297 (1508 / 1476).
+// H = 2048, V = 126464: of 2048 1536 418 / 429 (479 / 486); of 4096 4096 1084 / 1091 (1217 / 1235).
+// H = 1024, V = 100000: of 2048 1536 194 / 319, of 4096 4096 491 / 821.  H = 512, V = 30000: 2048
+// 72 / 128.
+// fdllm_lmhead_logits, which takes the same variant, H = 4096, V = 50000: 576 of 768 149 / 184, 768
+// of 1024 188 / 189, 1152 of 1536 291 / 286 (336 / 325); H = 1024, V = 30000, 1152 of 1536 62 / 108.
 // FDLLM_LMHEAD_GEMM = solo, pair, slab or wide forces one (slab only where B * L <= kSlabRows).
 constexpr int kWideDeepH = 2560;
-constexpr int kWideRowsMax = 4096;          // H <= kWideDeepH: the most rows measured
+constexpr int kWideRowsMax = 4096;          // H <= kWideDeepH: the most rows tried, no crossing point
 constexpr int kWideRowsDeep = 48 * 32;      // H beyond
 
 int gemm_mode(int64_t rows, int H, int V)
