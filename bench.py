@@ -489,9 +489,9 @@ def run_ours(args, rank: int, world: int, local_rank: int) -> dict | None:
 
 
 def run_e2e(args, torch, fd, w, sb) -> dict:
-    """The public call with page-locked host buffers: the host copies of the step's inputs
-    and results are inside the timed region (the masked rows are read by the GPU over the
-    host link, the rest copied)."""
+    """The public call with page-locked host buffers: the movement of the step's inputs and
+    results is inside the timed region (the masked rows are read by the GPU over the host link,
+    the mask is copied in, the results are written over the link)."""
     h_logits = torch.empty(sb.bufs[0].shape, dtype=sb.bufs[0].dtype, pin_memory=True)
     h_logits.copy_(sb.bufs[0])
     h_mask = torch.from_numpy(sb.mask0_np.copy()).pin_memory()
@@ -511,13 +511,12 @@ def run_e2e(args, torch, fd, w, sb) -> dict:
     t_e2e = time.perf_counter() - t0
     out = {"value": w.B * e2e_steps / t_e2e, "unit": UNIT,
            # only the masked rows cross the host link (read by the GPU from pinned memory)
-           "h2d_bytes_per_step": sb.masked_rows * w.V * w.elem_bytes
-           + h_mask.numel() + h_tok.numel() * 4,
+           "h2d_bytes_per_step": sb.masked_rows * w.V * w.elem_bytes + h_mask.numel(),
            "path": "fdllm_select_host (one C call): pinned host logits, the masked rows "
-                   "read by the GPU over the host link, mask and tokens copied in, the step, "
-                   "results and mask copied back",
-           "d2h_bytes_per_step": h_tok.numel() * 4 + h_commit.numel() + h_n.numel() * 4
-           + h_mask.numel(),
+                   "read by the GPU over the host link, the mask copied in, the step, whose "
+                   "selection writes the committed tokens, the commit flags and the counts "
+                   "to the pinned results over the link; the host clears its mask",
+           "d2h_bytes_per_step": int(h_n.sum()) * 4 + h_commit.numel() + h_n.numel() * 4,
            "steps": e2e_steps}
     del h_logits
     return out
