@@ -238,16 +238,16 @@ fdllm_status fdllm_gather_masked_rows(const void *src, void *dst, int dtype, int
  *           mask is updated in place and out_tokens keeps its values at positions not
  *           committed, as in fdllm_select.
  * The library copies the mask to a device staging buffer of its own (per device, grown on
- * demand with cudaMalloc, released by fdllm_release_workspace), runs the step on `stream`
- * with the library workspace and synchronises `stream` before it returns: the results are in
- * place when the call returns.  Where out_tokens, out_commit and out_n are page-locked and
- * the mask is in host memory, the step writes the three over the host link and the host
- * clears the committed positions of the mask after the synchronisation; otherwise out_tokens
- * is staged as well, and all four are copied back.  An array of which only a part is page-locked
- * is refused (FDLLM_ERR_CUDA: the runtime does not copy such a range).  Argument errors are reported before
- * anything is enqueued; the same device errors as fdllm_select (fdllm_device_status).  A call
- * that returns FDLLM_ERR_CUDA may have written page-locked results in part, and then leaves
- * the mask as it was.  Not for stream capture (it synchronises).
+ * demand with cudaMalloc, released by fdllm_release_workspace), runs the step on `stream` with
+ * the library workspace and synchronises `stream` before it returns: the results are in place
+ * when the call returns.  Where out_tokens, out_commit and out_n are page-locked and the mask
+ * is in host memory, the step writes the three over the host link and the host clears the
+ * committed positions of the mask after the synchronisation; otherwise out_tokens is staged as
+ * well, and all four are copied back.  An array of which only a part is page-locked is refused
+ * (FDLLM_ERR_CUDA: the runtime does not copy such a range).  Argument errors are reported
+ * before anything is enqueued; the same device errors as fdllm_select (fdllm_device_status).
+ * A call that returns FDLLM_ERR_CUDA may have written results in part, and then leaves the
+ * mask as it was.  Not for stream capture (it synchronises).
  * Calls share the staging buffer and the library workspace of their device: calls from
  * several host threads at once must be serialised by the caller.  The paper has no
  * counterpart. */
@@ -381,12 +381,12 @@ fdllm_status fdllm_profile_terms(const float *conf, const uint8_t *mask, int B, 
 fdllm_status fdllm_check_bounded_wait(double seconds, void *stream);
 
 /* Synchronises `stream`, then reports (and clears) the sticky device error of the library
- * workspace (and of those it outgrew) on the current device: FDLLM_ERR_DEVICE if a kernel gave up a bounded wait
- * since the last call, else FDLLM_ERR_NONFINITE if a selection since the last call found a
- * row of FDLLM_ROW_NONFINITE, FDLLM_OK otherwise.  For fdllm_select_ws, pass the workspace to
- * fdllm_workspace_status instead.  Clearing an error also resets the workspace's work
- * counter, which a launch that gave up may have left mid-queue, so that the next call
- * starts from a clean header. */
+ * workspace (and of those it outgrew) on the current device: FDLLM_ERR_DEVICE if a kernel gave
+ * up a bounded wait since the last call, else FDLLM_ERR_NONFINITE if a selection since the
+ * last call found a row of FDLLM_ROW_NONFINITE, FDLLM_OK otherwise.  For fdllm_select_ws, pass
+ * the workspace to fdllm_workspace_status instead.  Clearing an error also resets the
+ * workspace's work counter, which a launch that gave up may have left mid-queue, so that the
+ * next call starts from a clean header. */
 fdllm_status fdllm_device_status(void *stream);
 fdllm_status fdllm_workspace_status(void *workspace, void *stream);
 

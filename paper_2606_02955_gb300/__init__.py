@@ -211,9 +211,9 @@ def fdllm_select(logits: torch.Tensor, mask: torch.Tensor, param: float, mode=PR
     uint8 (updated in place).  Returns (out_tokens, out_commit, out_n).
 
     Device tensors run asynchronously on ``stream`` (default: current stream).  With host
-    tensors the call copies the inputs to the current CUDA device (pinned memory makes the
-    copies asynchronous), runs the step, copies the outputs and the updated mask back and
-    synchronises: the end-to-end form of the call."""
+    tensors the call is fdllm_select_host on the current CUDA device: the GPU reads the masked
+    rows of pinned logits (pageable ones are copied), the step runs, pinned outputs are written
+    in place (others copied back), the mask is updated, and the call synchronises."""
     if not logits.is_cuda:
         return _select_from_host(logits, mask, param, mode, out_tokens, out_commit, out_n)
     B, L, V = logits.shape
@@ -229,8 +229,7 @@ def fdllm_select(logits: torch.Tensor, mask: torch.Tensor, param: float, mode=PR
 
 
 def _select_from_host(logits, mask, param, mode, out_tokens, out_commit, out_n):
-    """fdllm_select_host: the whole step on host tensors in one library call (the GPU reads
-    only the masked rows of page-locked logits; results and mask copied back)."""
+    """fdllm_select_host: the whole step on host tensors in one library call."""
     B, L, V = logits.shape
     if not logits.is_contiguous():
         raise FdllmError(1, "fdllm_select_host: contiguous logits required")
