@@ -147,3 +147,33 @@ def test_graph_on_an_outgrown_workspace(fd):
     assert out[2].tolist()[1] == fd.ROW_NONFINITE
     assert fd.fdllm_device_status() == 0
     fd.fdllm_release_workspace()
+
+
+@pytest.mark.gpu
+def test_call_without_room_during_a_capture(fd):
+    """Refused on the host; the capture goes on, and so does the graph."""
+    fd.fdllm_release_workspace()
+    x = torch.randn(1, 32, 1000, device="cuda").to(torch.bfloat16)
+    mask = torch.ones(1, 32, dtype=torch.uint8, device="cuda")
+    conf, tok = fd.fdllm_confidence(x, mask)
+    big = torch.zeros(100, 32, 8, device="cuda", dtype=torch.bfloat16)
+    out = [torch.zeros(100, 32, dtype=t, device="cuda")
+           for t in (torch.uint8, torch.float32, torch.int32)]
+    c, t = torch.zeros_like(conf), torch.zeros_like(tok)
+
+    def calls():
+        with pytest.raises(fd.FdllmError) as e:
+            fd.fdllm_confidence(big, *out)
+        assert e.value.status == fd.ERR_CUDA
+        fd.fdllm_confidence(x, mask, c, t)
+
+    torch.cuda.synchronize()
+    g = _captured(calls)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(c, conf) and torch.equal(t, tok)
+    fd.fdllm_confidence(big, *out)  # grows now
+    assert fd.fdllm_device_status() == 0
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(c, conf) and fd.fdllm_device_status() == 0
