@@ -827,7 +827,7 @@ struct WidePiece {
 
 // The pieces of one CTA pair.  Whole rounds of items over the pairs first; if what is left then
 // fills at most half of them, each leftover item goes to two pairs, one group or half of the one
-// group each: halves of 96 and 64 columns (a group of 160) and up, since no narrower group was tried.
+// group each: halves of 96 and 64 columns (a group of 160) and up; no narrower group was tried.
 // Whole fdllm_lmhead_confidence pass with one-group items left whole against halved: 200 rows, H =
 // 4096, 20000 entries 49.5 -> 46.4 us, 65000 entries 98.7 -> 95.8, LLaDA's 169 -> 167; H = 1024,
 // 20000 entries 200 rows 20.6 -> 19.5, 700 rows 32.9 -> 31.4; H = 2048, 8000 entries 200 rows 19.5
@@ -1667,7 +1667,7 @@ int slab_grid(int V)
 // of 1024 188 / 189, 1152 of 1536 291 / 286 (336 / 325); H = 1024, V = 30000, 1152 of 1536 62 / 108.
 // FDLLM_LMHEAD_GEMM = solo, pair, slab or wide forces one (slab only where B * L <= kSlabRows).
 constexpr int kWideDeepH = 2560;
-constexpr int kWideRowsMax = 4096;          // H <= kWideDeepH: the most rows tried, no crossing point
+constexpr int kWideRowsMax = 4096;          // H <= kWideDeepH: the most rows measured
 constexpr int kWideRowsDeep = 48 * 32;      // H beyond
 
 int gemm_mode(int64_t rows, int H, int V)
